@@ -651,7 +651,7 @@ void bisect_body(bipart_graph *g, Level &L0, const Params &p, int64_t W, uint8_t
         run_tail(g, levels, p, limit, sa);
     }
     if (nlev) *nlev = (int)levels.size();
-    uncoarsen(g, levels, limit, p.m0, p.m, p.iters, d_side, tail_from);
+    uncoarsen(g, levels, limit, W, p.m0, p.m, p.iters, d_side, tail_from);
     prof_level(0, 0);
     if (g->ex.capturing) flush_checks(g);
 }
@@ -839,7 +839,7 @@ int refine_kept(bipart_graph *g, int64_t e6, int32_t iters, int *d_parts) {
         run_tail(g, levels, p, limit, sa);
     }
     if ((int)levels.size() != g->hier.nlev) throw Fail{BIPART_ERR_CUDA, "kept hierarchy changed size"};
-    uncoarsen(g, levels, limit, p.m0, p.m, p.iters, d_side, tail_from);
+    uncoarsen(g, levels, limit, W, p.m0, p.m, p.iters, d_side, tail_from);
     int st = read_bisect_status(g);
     k_side_to_part<<<grid_for(L0.N), kBlock, 0, s>>>(L0.N, d_side, nullptr, 0, p.m0, d_parts);
     BP_LAUNCH();

@@ -261,7 +261,7 @@ __device__ __noinline__ void blk_select_apply(Ctx &x, const DLevel &L, int kind,
     RState *st = x.st;
     unsigned(*h)[kHistBins] = reinterpret_cast<unsigned(*)[kHistBins]>(x.smem);
     if (L.N <= kSelOneBlock && L.N <= 32 * (int)blockDim.x) {
-        d_sel_small(L.N, kind, sq, x.gain, side, L.nw, st, x.status, x.list, nullptr, x.gain, x.grp, h);
+        d_sel_small(L.N, kind, sq, x.gain, side, L.nw, st, x.status, x.list, x.gain, x.grp, h);
         __syncthreads();
         return;
     }

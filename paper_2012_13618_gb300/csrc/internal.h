@@ -166,16 +166,12 @@ struct Work {
     Buf p_a;         // per-pin int32 scratch
     Buf side_a, side_b;      // uint8 sides (ping-pong across levels)
     Buf gain;        // int32 gains
-    Buf hc;          // int2 per-hyperedge gain contributions
-    Buf n1;          // int32 per-hyperedge side-1 pin counts: two halves used by alternate passes
-    int64_t n1_half = 0;
-    int64_t gain_pass = 0;   // gain passes so far in this bisection
-    int32_t n1_prev_E = 0;   // hyperedges counted by the previous pass (its half is dirty there)
-    const void *n1_level = nullptr;  // the level whose counts the current half holds (else null)
-    Buf moved;       // nodes moved since the counts were last brought up to date (int32)
+    Buf side_prev;   // uint8 sides before the last selection
+    Buf pair;        // uint64 pins on side 0 << 32 | pins on side 1 of every hyperedge
+    Buf ent;         // moved nodes' incidence runs
+    Buf items;       // work items of wide hyperedges whose contributions changed
     Buf e_best;      // per-hyperedge uint64 singleton-attach keys
     Buf m_fp, m_tkey, m_tmin, m_rep, m_wsum;  // parallel-net merging: fingerprints, table, groups
-    Buf partial;     // per-block partial sums of grid-wide reductions
     Buf list;        // node list (rebalance candidates)
     Buf pinned;      // host-pinned mirror of `small`
     uint32_t *host_small = nullptr;
@@ -388,12 +384,12 @@ int *degree_counters(bipart_graph *g, int32_t N);
 // Runs Algorithms 3, 5 (+ rebalance) over the hierarchy; writes side of level 0.  The status
 // (1 = the level-0 rebalance ran out of candidates) is left in *bisect_status_word(g).
 // Side 0 is meant for m0 of m parts: Algorithm 3 grows it to that share and limit[s] bounds
-// side s (halving bisection: m0 / m = 1 / 2, equal limits).
+// side s (halving bisection: m0 / m = 1 / 2, equal limits).  W: total node weight.
 // With tail_from >= 0 the levels from tail_from down were refined by the cluster tail, which left
 // the side of level tail_from in the handle's first side buffer (side_a).
-void uncoarsen(bipart_graph *g, std::vector<Level *> &levels, const int64_t limit[2], int m0,
+void uncoarsen(bipart_graph *g, std::vector<Level *> &levels, const int64_t limit[2], int64_t W, int m0,
                int m, int32_t iters, uint8_t *d_side0, int tail_from = -1);
-const unsigned *bisect_status_word(bipart_graph *g);
+unsigned *bisect_status_word(bipart_graph *g);
 // Bytes at the start of the small scratch holding counters and selection state that phases
 // leave zero for the next one (cleared once at the start of every bisection).
 size_t small_state_bytes();
@@ -418,8 +414,6 @@ void run_tail(bipart_graph *g, std::vector<Level *> &levels, const Params &p, co
               uint8_t *d_side);
 // Two device ints of the handle's size slots for the tail's level count and arena check.
 int32_t *tail_info_slot(bipart_graph *g);
-struct RState;
-RState *refine_state(bipart_graph *g);
 
 // ------------------------------------------------------------------------- diagnostics
 // Brackets one kernel launch with CUDA events on `s` when profiling is on (see

@@ -28,7 +28,7 @@ struct SelGroup {
     unsigned long long top;
 };
 
-// All device-side state of refinement, resident in the handle's small scratch.
+// The state of a level's selections, kept by the block (or by every block of a cluster alike).
 struct RState {
     SelGroup g[2];
     unsigned hist[2][kHistBins];
@@ -40,10 +40,6 @@ struct RState {
     unsigned slow;             // exact radix path needed by the current selection
     unsigned warn;             // rebalance ran out of candidates
     unsigned rounds;           // loop guard
-    unsigned status0;          // warn of the level-0 rebalance
-    unsigned arrived;          // blocks that finished a fused grid phase (zero at rest)
-    unsigned moved_count;      // nodes moved by the current selection (reset by each selection)
-    unsigned long long Wacc[2];  // side-weight partial sums of a grid launch (zero at rest)
 };
 
 __device__ __forceinline__ unsigned gkey(int gain) { return (unsigned)gain ^ 0x80000000u; }
@@ -56,68 +52,34 @@ __device__ __forceinline__ int sel_group(int kind, const RState *st, int gain, u
 }
 
 // ------------------------------------------------------------------------ Algorithm 4
-// n1[e] = number of pins of e on side 1 (load-balanced over pins, integer atomics).
+// Adds every hyperedge's side-1 pins to its pair (load-balanced over pins, 64-bit integer atomics).
+// pair[e] = pins on side 0 << 32 | pins on side 1, all pins counted on side 0 on entry.
 template <class Team>
 __device__ void d_hedge_n1(Team t, int E, int P, const int *hoff, const int *pins,
-                           const uint8_t *side, int *n1, const int *ts = nullptr) {
+                           const uint8_t *side, unsigned long long *pair, const int *ts = nullptr) {
     lb_for_each_items<int>(
         hoff, E, P, pins, 0,
         [&](int, int u, int acc) { return acc + Team::ld(side + u); },
         [&](int e, int acc) {
-            if (acc) atomicAdd(n1 + e, acc);
+            if (acc) atomicAdd(pair + e, (unsigned long long)acc * (1ull - (1ull << 32)));
         },
         t, ts);
 }
 
-// Contribution of e to a pin on side i: +w if n_i == 1 (moving it uncuts e), -w if n_i == |e|
-// (moving it cuts e), else 0.
-// With `reset`, n1[e] is put back to zero once read (the grid path keeps n1 zero at rest).
-template <class Team>
-__device__ void d_hedge_contrib(Team t, int E, const int *hoff, const int *hw, int *n1,
-                                int2 *hc, bool reset = false) {
-    for (int e = t.rank(); e < E; e += t.size()) {
-        int d = Team::ld(hoff + e + 1) - Team::ld(hoff + e), a1 = Team::ld(n1 + e), a0 = d - a1;
-        if (reset) n1[e] = 0;
-        int w = hw ? Team::ld(hw + e) : 1;
-        int c0 = a0 == 1 ? w : (a0 == d ? -w : 0);
-        int c1 = a1 == 1 ? w : (a1 == d ? -w : 0);
-        hc[e] = make_int2(c0, c1);
-    }
-}
-
-// gain[v] = sum over v's hyperedges of the contribution for v's side (gain zeroed first).
-template <class Team>
+// gain[v] = sum over v's hyperedges of their contribution to v's side (gain zeroed first): +w when
+// v is alone on it (moving it uncuts e), -w when e has no pin on the other (moving it cuts e).
 // With `warp_sum` the last runs of a warp's lanes are summed per node before the atomic (levels
 // whose nodes have long incidence lists, where many threads would hit one node).
-__device__ void d_node_gain(Team t, int N, int P, const int *noff, const int *nadj, const int2 *hc,
-                            const uint8_t *side, int *gain, const int *ts = nullptr,
-                            bool warp_sum = true) {
-    auto visit = [&](int v, int e, int acc) {
-        int2 c = Team::ld(hc + e);
-        return acc + (Team::ld(side + v) ? c.y : c.x);
-    };
-    auto flush = [&](int v, int acc) {
-        if (acc) atomicAdd(gain + v, acc);
-    };
-    if (warp_sum)
-        lb_reduce_items<int>(noff, N, P, nadj, 0, cooperative_groups::plus<int>(), visit, flush, t, ts);
-    else
-        lb_for_each_items<int>(noff, N, P, nadj, 0, visit, flush, t, ts);
-}
-
-// The same gains with each hyperedge's contribution formed on the spot from its degree, its
-// side-1 count and its weight (no separate contribution pass).
 template <class Team>
-__device__ void d_node_gain_direct(Team t, int N, int P, const int *noff, const int *nadj,
-                                   const int *hoff, const int *hw, const int *n1,
-                                   const uint8_t *side, int *gain, const int *ts = nullptr,
-                                   bool warp_sum = true) {
+__device__ void d_node_gain(Team t, int N, int P, const int *noff, const int *nadj,
+                            const unsigned long long *pair, const int *hw, const uint8_t *side, int *gain,
+                            const int *ts = nullptr, bool warp_sum = true) {
     auto visit = [&](int v, int e, int acc) {
-        const int d = Team::ld(hoff + e + 1) - Team::ld(hoff + e);
-        const int a1 = Team::ld(n1 + e);
-        const int w = hw ? Team::ld(hw + e) : 1;
-        const int a = Team::ld(side + v) ? a1 : d - a1;  // pins on v's side
-        return acc + (a == 1 ? w : (a == d ? -w : 0));
+        const unsigned long long q = Team::ld(pair + e);
+        const int n0 = (int)(q >> 32), n1 = (int)(unsigned)q;
+        const int own = Team::ld(side + v) ? n1 : n0, other = n0 + n1 - own;
+        const int c = (own == 1) - (other == 0);
+        return acc + (hw && c ? c * Team::ld(hw + e) : c);
     };
     auto flush = [&](int v, int acc) {
         if (acc) atomicAdd(gain + v, acc);
@@ -386,11 +348,9 @@ struct TieIn {
 };
 
 // Applies the selection to a chosen node v: refine flips it; the initial partition moves it to P0
-// and keeps the side weights current; the rebalance collects it.  With `moved`, every flipped node
-// is also appended there (st->moved_count; one atomic per group of converged lanes), so the
-// side-1 counts can be updated instead of recounted.
+// and keeps the side weights current; the rebalance collects it.
 __device__ __forceinline__ void d_apply_node(int kind, int64_t v, uint8_t *side, const int *nw,
-                                             RState *st, int *list, int *moved) {
+                                             RState *st, int *list) {
     if (kind == SEL_REBAL) {
         list[atomicAdd(&st->list_count, 1u)] = (int)v;
         return;
@@ -400,17 +360,9 @@ __device__ __forceinline__ void d_apply_node(int kind, int64_t v, uint8_t *side,
         atomicAdd(&st->W[0], (unsigned long long)nw[v]);
         atomicAdd(&st->W[1], (unsigned long long)(-(long long)nw[v]));
     }
-    if (moved) {
-        namespace cg = cooperative_groups;
-        const cg::coalesced_group grp = cg::coalesced_threads();
-        unsigned base = 0;
-        if (grp.thread_rank() == 0) base = atomicAdd(&st->moved_count, grp.size());
-        base = grp.shfl(base, 0);
-        moved[base + grp.thread_rank()] = (int)v;
-    }
 }
 
-// The application pass of a grid selection: the tie ranks come from the scan (TieIn).
+// The application pass of a selection: the tie ranks come from the scan (TieIn).
 struct ApplyOut {
     int kind;
     const int *gain;
@@ -418,7 +370,6 @@ struct ApplyOut {
     const int *nw;
     RState *st;
     int *list;
-    int *moved = nullptr;
     __device__ void operator()(int64_t v, uint64_t pre, uint64_t) const {
         int g = gain[v];
         int grp = sel_group(kind, st, g, side[v], nw[v]);
@@ -433,7 +384,7 @@ struct ApplyOut {
         } else {
             sel = false;
         }
-        if (sel) d_apply_node(kind, v, side, nw, st, list, moved);
+        if (sel) d_apply_node(kind, v, side, nw, st, list);
     }
 };
 
@@ -503,8 +454,7 @@ __device__ inline void d_rebal_cond(RState *st, long long limit0, long long limi
 // With nothing selected, marks the level imbalanced.  One block; keys: shared memory for the
 // next power of two >= the number selected.
 __device__ inline void d_rebal_move(const int *gain, uint8_t *side, const int *nw, const int *list,
-                                    RState *st, long long s, unsigned long long *keys,
-                                    int *moved = nullptr) {
+                                    RState *st, long long s, unsigned long long *keys) {
     __shared__ long long red[33];
     __shared__ int s_cut;
     const int n = (int)st->list_count;
@@ -561,13 +511,11 @@ __device__ inline void d_rebal_move(const int *gain, uint8_t *side, const int *n
         int v = (int)(keys[i] & 0xffffffffu);
         side[v] = (uint8_t)(1 - heavy);
         wmoved += nw[v];
-        if (moved) moved[i] = v;  // the selection that collected the candidates reset the count
     }
     wmoved = block_sum(wmoved, red);
     if (threadIdx.x == 0) {
         atomicAdd(&st->W[1 - heavy], (unsigned long long)wmoved);
         atomicAdd(&st->W[heavy], (unsigned long long)(-wmoved));
-        if (moved) st->moved_count = (unsigned)cut;
     }
 }
 
@@ -576,14 +524,13 @@ __device__ inline void d_rebal_move(const int *gain, uint8_t *side, const int *n
 // s_gain, s_grp: N entries each; s_gain may be `gain` itself when that is in shared memory), the
 // threshold (and the exact radix passes when it falls in a clamped end bucket), the ranks of the
 // threshold's ties by ascending id from a bitmap with per-word prefix counts, and the
-// application.  h: 2 x kHistBins counters.  The rebalancing list and the moved list are emptied
-// first.  Deterministic: the same inputs give the same sides in every block that runs it.
+// application.  h: 2 x kHistBins counters.  The rebalancing list is emptied first.  Deterministic: the same inputs give the same sides in every block that runs it.
 constexpr int kSelOneBlock = 16384;
 constexpr int kSelSmallWords = kSelOneBlock / 32;
 
 __device__ inline void d_sel_small(int N, int kind, long long s, const int *gain, uint8_t *side,
                                    const int *nw, RState *st, uint32_t *status, int *list,
-                                   int *moved, int *s_gain, signed char *s_grp,
+                                   int *s_gain, signed char *s_grp,
                                    unsigned (*h)[kHistBins]) {
     __shared__ unsigned tie[2][kSelSmallWords];
     __shared__ unsigned pre[2][kSelSmallWords];
@@ -603,10 +550,7 @@ __device__ inline void d_sel_small(int N, int kind, long long s, const int *gain
     });
     __syncthreads();
     d_sel_find(kind, s, st, h);
-    if (threadIdx.x == 0) {
-        st->list_count = 0;
-        st->moved_count = 0;
-    }
+    if (threadIdx.x == 0) st->list_count = 0;
     __syncthreads();
     if (*(volatile unsigned *)&st->slow) {
         for (int pass = 0; pass < 3; ++pass) {
@@ -655,7 +599,7 @@ __device__ inline void d_sel_small(int N, int kind, long long s, const int *gain
                 sel = pre[grp][v >> 5] + (unsigned)__popc(below) < s_take[grp];
             }
         }
-        if (sel) d_apply_node(kind, v, side, nw, st, list, moved);
+        if (sel) d_apply_node(kind, v, side, nw, st, list);
     }
 }
 

@@ -1,0 +1,82 @@
+// The refinement of one level as one thread-block-cluster launch (refine_loop.cu): its state in
+// the handle's small scratch, its arguments, and the pieces the grid kernels of a large level's
+// gain update share with it (move_dev.cuh).
+#pragma once
+
+#include <stdint.h>
+
+#include "refine_dev.cuh"
+
+namespace bp {
+
+constexpr int kLoopThreads = 512;       // threads per block of the cluster
+constexpr int kLoopMaxCluster = 16;
+constexpr int kMoveRun = 64;            // incidences of a moved node one entry of the move list covers
+constexpr int kItemPins = 512;          // pins of a wide hyperedge one work item covers
+constexpr int kItemCap = 1 << 16;       // work items a pass may queue (beyond: walked on the spot)
+// Moves of more than this many incidences are brought into the gains by the whole grid instead of
+// the one cluster (levels of more than kLoopAlonePins pins only; smaller ones stay in the cluster).
+constexpr long long kLoopMoveInc = 1 << 17;
+constexpr int64_t kLoopAlonePins = 1 << 18;
+// Levels of at most this many pins are started (sides projected, gains counted) by the cluster launch too.
+constexpr int kLoopStartPins = 1 << 17;
+// Levels of at most this many nodes are selected by the cluster's first block alone, the others helping
+// with the gain updates only.
+constexpr int kLoopSoloNodes = 4096;
+// Above P / kMoveFull moved incidences every gain is recomputed instead of updated.
+constexpr int kMoveFull = 8;
+
+// What one selection leaves for the update after it; two are used in turn.
+struct LoopRound {
+    unsigned ents, items, cands, pad;
+    unsigned long long inc;     // incidences of the moved nodes
+    unsigned long long weight;  // their node weight (initial partition)
+    unsigned ties[kLoopMaxCluster][2];
+};
+
+// Zero at the start of a level (k_level_start); lives in the handle's small scratch.
+struct LoopState {
+    unsigned hist[2][kHistBins];
+    LoopRound rd[2];
+    unsigned long long w1[kLoopMaxCluster];  // per-block sums of side 1's weight
+    unsigned cmd;      // next step of the helper blocks: 0 leave, else 1 | own << 1
+    unsigned pending;  // the launch stopped after a selection too large for one cluster
+    unsigned sel;      // which LoopRound the last selection used
+    unsigned it;       // refinement iterations done
+    unsigned status0;  // the level's rebalance ran out of candidates (the last level written is 0)
+    // a stop inside the rebalance: its state
+    unsigned rebal, rounds;
+    int heavy;
+    unsigned long long W[2];
+    long long room, need;
+};
+
+// A level's arrays as the gain update reads them.
+struct MoveArgs {
+    int N, E, P;
+    const int *noff, *nadj, *hoff, *pins, *hw, *nw;
+    uint8_t *side, *prev;
+    int *gain;
+    unsigned long long *pair;  // per hyperedge: pins on side 0 << 32 | pins on side 1
+    LoopState *ls;
+    int4 *ent;  // move list: node and its side now, incidences [y, z) (move_entry)
+    int4 *items;
+    int item_cap;
+    int lanes;  // lanes per entry of the move list (8 or 32)
+};
+
+struct LoopParams {
+    long long W, limit0, limit1, sq;
+    int m0, m, iters;
+    bool initial;  // Algorithm 3 first (all nodes on side 1)
+    bool resume;   // continue after the grid took a pending update
+    bool suspend;  // large moves may be left to the grid
+    bool start;    // the launch also projects the sides (from `coarse` by `cmap`) and counts the gains
+    const int *cmap;
+    const uint8_t *coarse;
+};
+void launch_refine_loop(cudaStream_t s, const MoveArgs &m, const LoopParams &p, unsigned long long *cand,
+                        uint32_t *status,
+                        unsigned *pending_slot);
+
+}  // namespace bp

@@ -922,7 +922,6 @@ __global__ void __launch_bounds__(kTT, 1) k_tail(TailArgs a) {
             if (threadIdx.x == 0) {
                 st->rounds = 0;
                 st->list_count = 0;
-                st->moved_count = 0;
                 st->slow = 0;
             }
             __syncthreads();
@@ -932,7 +931,7 @@ __global__ void __launch_bounds__(kTT, 1) k_tail(TailArgs a) {
             while (st->flag) {
                 tail_gains(a, L, ch, smem, R, side, l);
                 bytes += pass_bytes(L);
-                d_sel_small(L.N, SEL_INITIAL, sq, R.gf, side, L.nw, st, a.status, nullptr, nullptr, R.gf,
+                d_sel_small(L.N, SEL_INITIAL, sq, R.gf, side, L.nw, st, a.status, nullptr, R.gf,
                             s_grp, st->hist);
                 __syncthreads();
                 d_initial_cond(st, (long long)L.N + 1, a.status, false, a.m0, a.m);
@@ -958,7 +957,7 @@ __global__ void __launch_bounds__(kTT, 1) k_tail(TailArgs a) {
         for (int it = 0; it < a.iters; ++it) {
             tail_gains(a, L, ch, smem, R, side, l);
             bytes += pass_bytes(L);
-            d_sel_small(L.N, SEL_REFINE, 0, R.gf, side, L.nw, st, a.status, nullptr, nullptr, R.gf, s_grp,
+            d_sel_small(L.N, SEL_REFINE, 0, R.gf, side, L.nw, st, a.status, nullptr, R.gf, s_grp,
                         st->hist);
             __syncthreads();
             trace(a, l, 30);
@@ -969,7 +968,7 @@ __global__ void __launch_bounds__(kTT, 1) k_tail(TailArgs a) {
         while (st->flag) {
             tail_gains(a, L, ch, smem, R, side, l);
             bytes += pass_bytes(L);
-            d_sel_small(L.N, SEL_REBAL, sq, R.gf, side, L.nw, st, a.status, list, nullptr, R.gf, s_grp,
+            d_sel_small(L.N, SEL_REBAL, sq, R.gf, side, L.nw, st, a.status, list, R.gf, s_grp,
                         st->hist);
             __syncthreads();
             d_rebal_move(R.gf, side, L.nw, list, st, sq, keys);
@@ -983,7 +982,7 @@ __global__ void __launch_bounds__(kTT, 1) k_tail(TailArgs a) {
         const uint8_t *side = sides[cur];
         for (int v = threadIdx.x; v < a.N; v += kTT) a.side_out[v] = side[v];
         if (threadIdx.x == 0) {
-            a.gst->warn = st->warn;
+            *a.status0 = st->warn;
             a.info[2] = (int)((bytes + a.N) / 1024.0);  // KiB, with the side written
         }
     }
@@ -1085,7 +1084,7 @@ void run_tail(bipart_graph *g, std::vector<Level *> &levels, const Params &p, co
     a.sizes = level_sizes(g, sidx);
     a.info = tail_info_slot(g);
     a.side_out = d_side;
-    a.gst = refine_state(g);
+    a.status0 = bisect_status_word(g);
     a.status = dev_status(g);
     static const bool tracing = std::getenv("BIPART_TAIL_TRACE") != nullptr;
     a.trace = nullptr;

@@ -50,7 +50,7 @@ struct TailArgs {
     int *info;   // [0] new levels built, [1] MiB of arena a run needed but did not have,
                  // [2] algorithmic KiB the launch moved
     uint8_t *side_out;  // bisection of the starting level
-    RState *gst;        // the handle's refinement state: warn of the starting level's rebalance
+    unsigned *status0;  // whether the starting level's rebalance ran out of candidates
     uint32_t *status;
     unsigned long long *trace;  // diagnostics (BIPART_TAIL_TRACE, eager calls): phase time stamps
 };

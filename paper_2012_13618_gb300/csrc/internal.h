@@ -221,7 +221,6 @@ struct Exec {
     uint64_t rec_gen = 0;
     int rec_nlev = 0;
     int64_t rec_kernels = 0;
-    bool rec_tail = false;  // the recorded run used the cluster tail (not captured: see bisect_top)
 };
 
 struct Probe {
@@ -353,8 +352,7 @@ struct bipart_graph {
     // budget): with one lane, the top bisection's coarse levels before the subgraphs'
     bool lean = false;
     bool ext_alloc = false;  // some buffer of this handle came from a bipart_set_allocator hook
-    int32_t last_tail_from = -1;
-    bool allow_tail = true;  // the next bisection may hand its coarse levels to the cluster tail  // tail start of the last bisection run on the host (eager or captured)
+    int32_t last_tail_from = -1;  // tail start of the last bisection run on the host (eager or captured)
     ~bipart_graph();
 };
 
@@ -389,7 +387,10 @@ int *degree_counters(bipart_graph *g, int32_t N);
 // the side of level tail_from in the handle's first side buffer (side_a).
 void uncoarsen(bipart_graph *g, std::vector<Level *> &levels, const int64_t limit[2], int64_t W, int m0,
                int m, int32_t iters, uint8_t *d_side0, int tail_from = -1);
+// A buffer of n sides, aligned for the four-nodes-at-a-time loads of the refinement whatever the allocator.
+uint8_t *side_buffer(Buf &b, int64_t n, cudaStream_t s);
 unsigned *bisect_status_word(bipart_graph *g);
+unsigned long long *bisect_weights(bipart_graph *g);  // the side weights of the level last refined
 // Bytes at the start of the small scratch holding counters and selection state that phases
 // leave zero for the next one (cleared once at the start of every bisection).
 size_t small_state_bytes();
@@ -410,7 +411,7 @@ bool tail_eligible(const Level &L, int max_new, int flags);
 // Runs the tail from levels.back(): appends the coarse levels it builds (arena views in g->lev),
 // writes the bisection of the starting level to d_side and its rebalance status to the handle's
 // refinement state.  Eager: one launch and one size read-back; while capturing: the recorded sizes.
-void run_tail(bipart_graph *g, std::vector<Level *> &levels, const Params &p, const int64_t limit[2],
+void run_tail(bipart_graph *g, std::vector<Level *> &levels, const Params &p, const int64_t limit[2], int64_t W,
               uint8_t *d_side);
 // Two device ints of the handle's size slots for the tail's level count and arena check.
 int32_t *tail_info_slot(bipart_graph *g);

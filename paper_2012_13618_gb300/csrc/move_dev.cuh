@@ -28,7 +28,9 @@
 
 namespace bp {
 
-constexpr int kWalkThread = 32;  // hyperedges up to this degree are walked by one thread
+constexpr int kWalkThread = 32;  // long lists: hyperedges up to this degree are walked by one thread,
+constexpr int kWalkWarp = 512;   // up to this one by the warp that met them, wider ones queued
+constexpr int kWalkShort = 8;    // short lists: wider ones are all queued, so that no warp walks several
 
 __device__ __forceinline__ int contrib(int own, int other) { return (own == 1) - (other == 0); }
 
@@ -43,8 +45,9 @@ __device__ __forceinline__ int4 move_entry(int v, int b, int d, int q, int s) {
 }
 
 // Adds x0 / x1 to the gains of pins [a, b) on side 0 / 1 of `wside`; thread `t` of `nt`.
-__device__ __forceinline__ void walk_pins(const int *pins, const uint8_t *wside, int *gain, int a, int b,
+static __device__ __noinline__ void walk_pins(const int *pins, const uint8_t *wside, int *gain, int a, int b,
                                           int x0, int x1, int t, int nt) {
+#pragma unroll 1
     for (int i0 = a + t; i0 < b; i0 += 4 * nt) {
         int u[4], s[4];
 #pragma unroll
@@ -62,7 +65,7 @@ __device__ __forceinline__ void walk_pins(const int *pins, const uint8_t *wside,
 // Pass 1 over the move list's n entries by warps [warp, warps).  queued: the count of work items (zero
 // before the pass).  wside: the sides the walked pins are read by (prev, or the current sides when moved
 // nodes' gains are not needed any more).  With `full` only the pairs are brought up to date.
-__device__ inline void move_pass1(const MoveArgs &m, unsigned n, unsigned *queued, int warp, int warps,
+static __device__ __noinline__ void move_pass1(const MoveArgs &m, unsigned n, unsigned *queued, int warp, int warps,
                                   const uint8_t *wside, bool full) {
     const int lane = threadIdx.x & 31;
     const int per = 32 / m.lanes, sub = lane % m.lanes, slot = lane / m.lanes;
@@ -79,6 +82,7 @@ __device__ inline void move_pass1(const MoveArgs &m, unsigned n, unsigned *queue
             step = pair_step(en.w);
         }
         if (full) {
+#pragma unroll 4
             for (; j < jb; j += m.lanes) atomicAdd(m.pair + __ldg(m.nadj + j), step);
             continue;
         }
@@ -99,28 +103,28 @@ __device__ inline void move_pass1(const MoveArgs &m, unsigned n, unsigned *queue
                     x1 *= w;
                 }
             }
-            if (d > 0 && d <= kWalkThread) walk_pins(m.pins, wside, m.gain, a, a + d, x0, x1, 0, 1);
-            unsigned wide = __ballot_sync(0xffffffffu, d > kWalkThread);
+            if (d > 0 && d <= (early ? kWalkShort : kWalkThread)) walk_pins(m.pins, wside, m.gain, a, a + d, x0, x1, 0, 1);
+            // wide hyperedges queued for pass 2, one place per kItemPins pins
+            const unsigned items = d > (early ? kWalkShort : kWalkWarp) ? (unsigned)(d + kItemPins - 1) / kItemPins : 0u;
+            if (__any_sync(0xffffffffu, items != 0)) {
+                const unsigned upto = warp_inclusive_scan(items);
+                unsigned base = 0;
+                if (lane == 31) base = atomicAdd(queued, upto);
+                base = __shfl_sync(0xffffffffu, base, 31) + upto - items;
+#pragma unroll 1
+                for (unsigned i = 0; i < items; ++i) {
+                    const int p0 = a + (int)i * kItemPins, p1 = min(p0 + kItemPins, a + d);
+                    if (base + i < (unsigned)m.item_cap) m.items[base + i] = make_int4(p0, p1, x0, x1);
+                    else walk_pins(m.pins, wside, m.gain, p0, p1, x0, x1, 0, 1);  // a full queue
+                }
+            }
+            unsigned wide = early ? 0u : __ballot_sync(0xffffffffu, d > kWalkThread && d <= kWalkWarp);
             while (wide) {
                 const int src = __ffs(wide) - 1;
                 wide &= wide - 1;
                 const int wa = __shfl_sync(0xffffffffu, a, src), wd = __shfl_sync(0xffffffffu, d, src);
                 const int y0 = __shfl_sync(0xffffffffu, x0, src), y1 = __shfl_sync(0xffffffffu, x1, src);
-                if (wd > kItemPins) {
-                    const int items = (wd + kItemPins - 1) / kItemPins;
-                    unsigned base = 0;
-                    if (lane == 0) base = atomicAdd(queued, (unsigned)items);
-                    base = __shfl_sync(0xffffffffu, base, 0);
-                    for (int i = lane; i < items; i += 32)
-                        if (base + i < (unsigned)m.item_cap)
-                            m.items[base + i] = make_int4(wa + i * kItemPins, min(wa + (i + 1) * kItemPins, wa + wd), y0, y1);
-                    // a full queue: the part that does not fit is walked here
-                    const int kept = base >= (unsigned)m.item_cap ? 0 : min(items, m.item_cap - (int)base);
-                    if (kept < items)
-                        walk_pins(m.pins, wside, m.gain, wa + kept * kItemPins, wa + wd, y0, y1, lane, 32);
-                } else {
-                    walk_pins(m.pins, wside, m.gain, wa, wa + wd, y0, y1, lane, 32);
-                }
+                walk_pins(m.pins, wside, m.gain, wa, wa + wd, y0, y1, lane, 32);
             }
             j += m.lanes;
         }
@@ -128,10 +132,11 @@ __device__ inline void move_pass1(const MoveArgs &m, unsigned n, unsigned *queue
 }
 
 // Pass 2: the queued items, and with `own` the moved nodes' corrections.
-__device__ inline void move_pass2(const MoveArgs &m, unsigned n, unsigned queued, int warp, int warps,
+static __device__ __noinline__ void move_pass2(const MoveArgs &m, unsigned n, unsigned queued, int warp, int warps,
                                   const uint8_t *wside, bool own) {
     const int lane = threadIdx.x & 31;
     const int items = (int)min(queued, (unsigned)m.item_cap);
+#pragma unroll 1
     for (int i = warp; i < items; i += warps) {
         const int4 it = __ldcg(m.items + i);
         walk_pins(m.pins, wside, m.gain, it.x, it.y, it.z, it.w, lane, 32);
@@ -154,13 +159,15 @@ __device__ inline void move_pass2(const MoveArgs &m, unsigned n, unsigned queued
                 if (x) acc += m.hw ? x * __ldg(m.hw + e) : x;
             }
         }
+#pragma unroll 1
         for (int o = m.lanes >> 1; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o, m.lanes);
         if (sub == 0 && acc) atomicAdd(m.gain + v, acc);
     }
 }
 
 // prev brought up to date for the moved nodes, before the next selection's update.
-__device__ inline void move_settle(const MoveArgs &m, unsigned n, int rank, int size) {
+static __device__ __noinline__ void move_settle(const MoveArgs &m, unsigned n, int rank, int size) {
+#pragma unroll 2
     for (unsigned k = (unsigned)rank; k < n; k += (unsigned)size) {
         const int4 en = __ldcg(m.ent + k);
         m.prev[en.x] = (uint8_t)en.w;

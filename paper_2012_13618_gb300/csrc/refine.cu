@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstddef>
 
 #include "common.cuh"
 #include "internal.h"
@@ -31,6 +32,11 @@
 namespace bp {
 
 namespace {
+
+template <class T>
+T *align16(T *p) {
+    return reinterpret_cast<T *>((reinterpret_cast<uintptr_t>(p) + 15) & ~uintptr_t(15));
+}
 
 constexpr int kBlock = 256;
 
@@ -63,7 +69,7 @@ k_level_start(int N, int E, const int *__restrict__ cmap, const uint8_t *__restr
         if (i < E) pair[i] = (unsigned long long)(unsigned)(__ldg(hoff + i + 1) - __ldg(hoff + i)) << 32;
     }
     if (blockIdx.x == 0)
-        for (int i = threadIdx.x; i < (int)(sizeof(LoopState) / sizeof(unsigned)); i += blockDim.x)
+        for (int i = threadIdx.x; i < (int)(offsetof(LoopState, cmd) / sizeof(unsigned)); i += blockDim.x)
             reinterpret_cast<unsigned *>(ls)[i] = 0;
 }
 
@@ -145,8 +151,8 @@ void refine_level(bipart_graph *g, Level &L, const int *cmap, const uint8_t *coa
     m.N = L.N; m.E = L.E; m.P = L.P;
     m.noff = L.noff(); m.nadj = L.nadj(); m.hoff = L.hoff(); m.pins = L.pins(); m.hw = L.hw(); m.nw = L.nw();
     m.side = side;
-    m.prev = w.side_prev.as<uint8_t>();
-    m.gain = w.gain.as<int>();
+    m.prev = align16(w.side_prev.as<uint8_t>());
+    m.gain = align16(w.gain.as<int>());
     m.pair = w.pair.as<unsigned long long>();
     m.ls = ls;
     m.ent = w.ent.as<int4>();
@@ -215,10 +221,10 @@ void uncoarsen(bipart_graph *g, std::vector<Level *> &levels, const int64_t limi
         pmax = std::max<int64_t>(pmax, levels[l]->P);
     }
     Work &w = g->w;
-    uint8_t *sa = (uint8_t *)w.side_a.ensure((size_t)nmax, s);
-    uint8_t *sb = (uint8_t *)w.side_b.ensure((size_t)nmax, s);
-    w.side_prev.ensure((size_t)nmax, s);
-    w.gain.ensure(sizeof(int) * (size_t)nmax, s);
+    uint8_t *sa = side_buffer(w.side_a, nmax, s);
+    uint8_t *sb = side_buffer(w.side_b, nmax, s);
+    side_buffer(w.side_prev, nmax, s);
+    w.gain.ensure(sizeof(int) * (size_t)nmax + 16, s);
     w.pair.ensure(sizeof(unsigned long long) * (size_t)emax, s);
     w.ent.ensure(sizeof(int4) * (size_t)(nmax + pmax / kMoveRun + 1), s);
     w.items.ensure(sizeof(int4) * (size_t)kItemCap, s);
@@ -244,7 +250,11 @@ void uncoarsen(bipart_graph *g, std::vector<Level *> &levels, const int64_t limi
         BP_CUDA(cudaMemcpyAsync(d_side0, cur, (size_t)levels[0]->N, cudaMemcpyDeviceToDevice, s));
 }
 
+uint8_t *side_buffer(Buf &b, int64_t n, cudaStream_t s) { return align16((uint8_t *)b.ensure((size_t)n + 16, s)); }
+
 unsigned *bisect_status_word(bipart_graph *g) { return &loop_state(g)->status0; }
+
+unsigned long long *bisect_weights(bipart_graph *g) { return loop_state(g)->W; }
 
 size_t small_state_bytes() { return 256 + sizeof(LoopState); }
 

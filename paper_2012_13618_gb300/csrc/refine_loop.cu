@@ -33,6 +33,7 @@
 #include "internal.h"
 #include "move_dev.cuh"
 #include "refine_loop.h"
+#include "select_dev.cuh"
 
 namespace bp {
 
@@ -63,19 +64,48 @@ constexpr int kStep = 8 * kT;            // nodes a block visits between two flu
 constexpr int kChosenCap = kStep + 4096;
 constexpr int kHubs = 64;                // chosen nodes whose long entry lists the block writes together
 
+// The block's view of a launch.  Solo: this block selects for the whole level (the other blocks of the
+// cluster only help with the gain updates).
+struct Ctx {
+    int r, C, lo, hi;
+    bool solo;
+    bool wvec;                   // the weights are aligned for 16-byte loads (the other node arrays are)
+    int p;                       // LoopRound of the last selection
+};
+
+// What the threshold leaves to decide: a group's mode and threshold gain, and whether some of its ties stay.
+struct Taken {
+    unsigned mode[2], thr[2];
+    bool some[2], hit;
+    // 2: taken, 1: a tie to be ranked, 0: not taken
+    __device__ __forceinline__ int operator()(int grp, int g) const {
+        const unsigned k = gkey(g), md = grp ? mode[1] : mode[0], th = grp ? thr[1] : thr[0];
+        if (md == 1) return 2;
+        if (md != 2 || k < th) return 0;
+        if (k > th) return 2;
+        if (hit) return 0;  // in the bitmap already
+        return (grp ? some[1] : some[0]) ? 1 : 2;
+    }
+};
+
+// Everything the phases share, the launch's arguments among it: they are functions of their own with plain
+// arguments, since what is passed by value or reference goes through each thread's stack.
 struct Shared {
-    LoopArgs a;                  // the launch's arguments (functions below are not inlined)
+    LoopArgs a;
+    Ctx x;
+    unsigned long long inc, weight;  // of the selection at hand (LoopRound)
     int guessed, guess;          // rebalance: the last round's threshold gain, if there is one
     LoopRound rd;                // solo: the round's counters
     alignas(16) RState st;       // this block's copy of the selection state; st.hist: its histogram
-    unsigned long long red[33];
+    unsigned red[32];
     int2 chosen[kChosenCap];     // nodes taken and the side they move to (rebalance candidates: their gain)
     unsigned nlist, nchosen, nhub, base;
     int2 hub[kHubs];
     unsigned hub_at[kHubs];
-    unsigned wsum[2][kWarps], bin[2], above[2], ntie[2], slow;
-    int cut;
-    long long moved;
+    unsigned ntie[2];
+    FindScratch find;
+    Taken taken;
+    CutScratch cut;
     // the rebalance's sort keys take the place of what follows (and may reach past it)
     alignas(16) unsigned bits[2][kWinWords];  // the threshold's ties per group, one bit per node of the window
     int2 list[kListCap];         // candidates (node | group << 31, gain)
@@ -91,26 +121,20 @@ __device__ __forceinline__ Shared &sh() {
     return *reinterpret_cast<Shared *>(smem);
 }
 
-// The block's view of a launch.  Solo: this block selects for the whole level (the other blocks of the
-// cluster only help with the gain updates).
-struct Ctx {
-    int r, C, lo, hi;
-    bool solo;
-    bool vec;                    // node arrays aligned for 16-byte loads
-    int p;                       // LoopRound of the last selection
-    __device__ LoopRound *rd() const { return solo ? &sh().rd : &sh().a.m.ls->rd[p]; }
-    // a counter of the round, after a barrier of the selecting blocks
-    template <class T>
-    __device__ __forceinline__ T count(T LoopRound::*f) const { return solo ? sh().rd.*f : __ldcg(&(sh().a.m.ls->rd[p].*f)); }
-    __device__ void sync() const {  // all blocks of the cluster
-        if (C == 1) __syncthreads();
-        else cg::this_cluster().sync();
-    }
-    __device__ void sel_sync() const {  // the selecting blocks
-        if (solo) __syncthreads();
-        else sync();
-    }
-};
+__device__ __forceinline__ void cluster_sync() {  // all blocks of the cluster
+    if (sh().x.C == 1) __syncthreads();
+    else cg::this_cluster().sync();
+}
+__device__ __forceinline__ void sel_sync() {  // the selecting blocks
+    if (sh().x.solo) __syncthreads();
+    else cluster_sync();
+}
+__device__ __forceinline__ LoopRound *global_round() { return &sh().a.m.ls->rd[sh().x.p]; }
+// A counter of the round, after a barrier of the selecting blocks.
+template <class T>
+__device__ __forceinline__ T round_count(T LoopRound::*f) {
+    return sh().x.solo ? sh().rd.*f : __ldcg(&(global_round()->*f));
+}
 
 // A step's eight nodes of a thread: two quads of consecutive nodes; slots of nodes that do not exist
 // hold the lowest gain.
@@ -123,11 +147,13 @@ struct Step {
 };
 
 // fn(step) for the nodes [lo, hi) of the block, kStep nodes per step, by all threads, converged.  The gains
-// are loaded first, then the sides and weights of the quads that have a node of at least `floor`.
+// are loaded first, then the sides and weights of the quads that have a node of at least `floor`.  The quad
+// at the end of a range is loaded whole (the arrays have slack).
 template <class Fn>
-__device__ __forceinline__ void visit_nodes(const Ctx &x, int lo, int hi, int floor, bool need_w,
+__device__ __forceinline__ void visit_nodes(int lo, int hi, int floor, bool need_w,
                                             const uint8_t *sides, Fn fn) {
     const int *gain = sh().a.m.gain, *nw = sh().a.m.nw;
+#pragma unroll 1
     for (int v0 = lo; v0 < hi; v0 += kStep) {
         Step t;
         t.v0 = v0;
@@ -135,33 +161,22 @@ __device__ __forceinline__ void visit_nodes(const Ctx &x, int lo, int hi, int fl
         for (int u = 0; u < 2; ++u) {
             const int v = t.node(4 * u);
             int4 g = make_int4(INT_MIN, INT_MIN, INT_MIN, INT_MIN);
-            if (v + 3 < hi && x.vec) {
-                g = __ldcg(reinterpret_cast<const int4 *>(gain + v));
-            } else if (v < hi) {
-                g.x = __ldcg(gain + v);
-                if (v + 1 < hi) g.y = __ldcg(gain + v + 1);
-                if (v + 2 < hi) g.z = __ldcg(gain + v + 2);
-                if (v + 3 < hi) g.w = __ldcg(gain + v + 3);
-            }
-            t.g[4 * u] = g.x; t.g[4 * u + 1] = g.y; t.g[4 * u + 2] = g.z; t.g[4 * u + 3] = g.w;
+            if (v < hi) g = __ldcg(reinterpret_cast<const int4 *>(gain + v));
+            t.g[4 * u] = g.x;
+            t.g[4 * u + 1] = v + 1 < hi ? g.y : INT_MIN;
+            t.g[4 * u + 2] = v + 2 < hi ? g.z : INT_MIN;
+            t.g[4 * u + 3] = v + 3 < hi ? g.w : INT_MIN;
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int v = t.node(4 * u);
             int4 w = make_int4(0, 0, 0, 0);
             t.sd[u] = 0;
-            if (v < hi && max(max(t.g[4 * u], t.g[4 * u + 1]), max(t.g[4 * u + 2], t.g[4 * u + 3])) >= floor) {
-                if (v + 3 < hi && x.vec) {
-                    t.sd[u] = __ldcg(reinterpret_cast<const unsigned *>(sides + v));
-                    if (need_w) w = __ldg(reinterpret_cast<const int4 *>(nw + v));
-                } else {
-                    for (int k = 0; k < 4 && v + k < hi; ++k) t.sd[u] |= (unsigned)__ldcg(sides + v + k) << (8 * k);
-                    if (need_w) {
-                        w.x = __ldg(nw + v);
-                        if (v + 1 < hi) w.y = __ldg(nw + v + 1);
-                        if (v + 2 < hi) w.z = __ldg(nw + v + 2);
-                        if (v + 3 < hi) w.w = __ldg(nw + v + 3);
-                    }
+            if (max(max(t.g[4 * u], t.g[4 * u + 1]), max(t.g[4 * u + 2], t.g[4 * u + 3])) >= floor) {
+                t.sd[u] = __ldcg(reinterpret_cast<const unsigned *>(sides + v));
+                if (need_w) {
+                    if (sh().x.wvec) w = __ldg(reinterpret_cast<const int4 *>(nw + v));
+                    else w = make_int4(__ldg(nw + v), __ldg(nw + v + 1), __ldg(nw + v + 2), __ldg(nw + v + 3));
                 }
             }
             t.w[4 * u] = w.x; t.w[4 * u + 1] = w.y; t.w[4 * u + 2] = w.z; t.w[4 * u + 3] = w.w;
@@ -195,19 +210,23 @@ __device__ __forceinline__ unsigned warp_places(unsigned *count, unsigned n) {
 
 // The chosen nodes join the level's lists: the rebalance's candidates, or (flipped already) the move
 // list, one entry per kMoveRun incidences and at least one per node.  All threads.
-__device__ __noinline__ void flush_chosen(const Ctx x, int kind, unsigned long long &inc, unsigned long long &weight) {
+__device__ __noinline__ void flush_chosen(int kind) {
     Shared &s = sh();
     const MoveArgs &m = s.a.m;
+    unsigned inc = 0;
+    int weight = 0;
     __syncthreads();
     const int n = (int)s.nchosen;
     if (n == 0) return;  // block-uniform
     if (kind == SEL_REBAL) {
-        if (x.solo) return;  // at most ceil(sqrt kLoopSoloNodes) of them: they stay in shared memory
-        if (threadIdx.x == 0) s.base = atomicAdd(&x.rd()->cands, (unsigned)n);
+        if (s.x.solo) return;  // at most ceil(sqrt kLoopSoloNodes) of them: they stay in shared memory
+        if (threadIdx.x == 0) s.base = atomicAdd(&global_round()->cands, (unsigned)n);
         __syncthreads();
+#pragma unroll 1
         for (int i = threadIdx.x; i < n; i += kT)
             s.a.cand[s.base + i] = (unsigned long long)~gkey(s.chosen[i].y) << 32 | (unsigned)s.chosen[i].x;
     } else {
+#pragma unroll 1
         for (int i0 = 0; i0 < n; i0 += kT) {
             const int i = i0 + (int)threadIdx.x;
             int v = 0, sd = 0, b = 0, d = 0, c = 0;
@@ -217,17 +236,23 @@ __device__ __noinline__ void flush_chosen(const Ctx x, int kind, unsigned long l
                 b = __ldg(m.noff + v);
                 d = __ldg(m.noff + v + 1) - b;
                 inc += (unsigned)d;
-                if (kind == SEL_INITIAL) weight += (unsigned)__ldg(m.nw + v);
+                const int w = __ldg(m.nw + v);
+                weight += sd ? w : -w;
                 c = d > 0 ? (d + kMoveRun - 1) / kMoveRun : 1;
             }
-            unsigned long long tot;
-            const unsigned long long ex = block_exclusive_scan<unsigned long long>((unsigned long long)c, s.red, &tot);
+            unsigned tot;
+            const unsigned ex = block_scan32<kT>((unsigned)c, s.red, &tot);
             if (threadIdx.x == 0) {
-                s.base = atomicAdd(&x.rd()->ents, (unsigned)tot);
+                if (s.x.solo) {
+                    s.base = s.rd.ents;
+                    s.rd.ents += tot;
+                } else {
+                    s.base = atomicAdd(&global_round()->ents, tot);
+                }
                 s.nhub = 0;
             }
             __syncthreads();
-            const unsigned o = s.base + (unsigned)ex;
+            const unsigned o = s.base + ex;
             bool mine = c > 0;
             if (c > 8) {
                 const unsigned h = atomicAdd(&s.nhub, 1u);
@@ -238,19 +263,43 @@ __device__ __noinline__ void flush_chosen(const Ctx x, int kind, unsigned long l
                 }
             }
             if (mine)
+#pragma unroll 1
                 for (int q = 0; q < c; ++q) m.ent[o + q] = move_entry(v, b, d, q, sd);
             __syncthreads();
             const int hubs = (int)min(s.nhub, (unsigned)kHubs);
+#pragma unroll 1
             for (int h = 0; h < hubs; ++h) {
                 const int hv = s.hub[h].x, hb = __ldg(m.noff + hv), hd = __ldg(m.noff + hv + 1) - hb;
+#pragma unroll 1
                 for (int q = threadIdx.x; q * kMoveRun < hd; q += kT) m.ent[s.hub_at[h] + q] = move_entry(hv, hb, hd, q, s.hub[h].y);
             }
             __syncthreads();
         }
     }
+    // a block's share of the incidences stays below 2^31, a warp's of one flush as well
+    inc = __reduce_add_sync(0xffffffffu, inc);
+    weight = __reduce_add_sync(0xffffffffu, weight);
+    if ((threadIdx.x & 31) == 0) {
+        if (inc) atomicAdd(&s.inc, (unsigned long long)inc);
+        if (weight) atomicAdd(&s.weight, (unsigned long long)(long long)weight);
+    }
     __syncthreads();
     if (threadIdx.x == 0) s.nchosen = 0;
     __syncthreads();
+}
+
+// The round's sums of this block's flushes (thread 0, after a flush) join its counters.
+__device__ __forceinline__ void add_sums() {
+    Shared &s = sh();
+    if (s.x.solo) {
+        s.rd.inc += s.inc;
+        s.rd.weight += s.weight;
+    } else {
+        LoopRound *rd = global_round();
+        if (s.inc) atomicAdd(&rd->inc, s.inc);
+        if (s.weight) atomicAdd(&rd->weight, s.weight);
+    }
+    s.inc = s.weight = 0;
 }
 
 // A node taken by the selection, in place `o` of the chosen: flipped (refinement, initial partition) or a
@@ -261,21 +310,25 @@ __device__ __forceinline__ void choose(int kind, unsigned o, int v, int side, in
 }
 
 // The block's histogram becomes the selecting blocks' total.
-__device__ __noinline__ void sum_hist(const Ctx x) {
+__device__ __noinline__ void sum_hist() {
     __syncthreads();
-    if (x.solo) return;
+    if (sh().x.solo) return;
     unsigned *h = &sh().st.hist[0][0], *g = &sh().a.m.ls->hist[0][0];
+#pragma unroll 1
     for (int i = threadIdx.x; i < 2 * kHistBins; i += kT)
         if (h[i]) atomicAdd(g + i, h[i]);
-    x.sync();
+    cluster_sync();
+#pragma unroll 2
     for (int i = threadIdx.x; i < kHistBins / 2; i += kT)
         reinterpret_cast<uint4 *>(h)[i] = __ldcg(reinterpret_cast<const uint4 *>(g) + i);
     __syncthreads();
 }
 
 __device__ __forceinline__ void clear_pass(int words) {
+#pragma unroll 1
     for (int i = threadIdx.x; i < kHistBins / 2; i += kT)
         reinterpret_cast<uint4 *>(&sh().st.hist[0][0])[i] = make_uint4(0, 0, 0, 0);
+#pragma unroll 1
     for (int i = threadIdx.x; i < words; i += kT) sh().bits[0][i] = sh().bits[1][i] = 0;
     if (threadIdx.x == 0) {
         sh().nlist = 0;
@@ -284,124 +337,25 @@ __device__ __forceinline__ void clear_pass(int words) {
     __syncthreads();
 }
 
-// d_sel_find's decision from the histogram's totals with three barriers: a warp sums 128 bins, every
-// warp scans the sums, the warp holding the threshold searches its bins.  With a guess, `ties`
-// candidates sit at the guessed gain and the histogram holds those above it; returns false when the
-// threshold lies below the guess.
-__device__ __noinline__ bool find_threshold(int kind, bool guess, unsigned ties) {
-    const long long sq = sh().a.sq;
-    Shared &s = sh();
-    RState *st = &s.st;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int kPer = kHistBins / kT;
-    static_assert(kPer == 4, "one uint4 of bins per thread and group");
-    const int b0 = kHistBins - kPer * ((int)threadIdx.x + 1);  // this thread's bins, from the highest down
-    uint4 c[2];
-    unsigned own[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        c[i] = *reinterpret_cast<const uint4 *>(&st->hist[i][b0]);
-        own[i] = c[i].x + c[i].y + c[i].z + c[i].w;
-        const unsigned w = __reduce_add_sync(0xffffffffu, own[i]);
-        if (lane == 0) s.wsum[i][wid] = w;
-    }
-    if (threadIdx.x < 2) s.bin[threadIdx.x] = ~0u;
-    if (threadIdx.x == 0) s.slow = 0;
-    __syncthreads();
-    unsigned cnt[2], before[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const unsigned inc = warp_inclusive_scan(lane < kWarps ? s.wsum[i][lane] : 0u);
-        cnt[i] = __shfl_sync(0xffffffffu, inc, 31);
-        before[i] = wid ? __shfl_sync(0xffffffffu, inc, wid - 1) : 0u;
-    }
-    const int heavy = st->heavy;
-    bool hit = false;
-    unsigned K[2] = {0, 0};
-    if (kind == SEL_REFINE) {
-        K[0] = K[1] = min(cnt[0], cnt[1]);
-    } else {
-        const int grp = kind == SEL_INITIAL ? 1 : heavy;
-        const unsigned have = grp >= 0 ? cnt[grp] : 0u;
-        if (guess && (long long)have < sq) {
-            if ((long long)have + ties < sq) return false;  // the same in every thread and block
-            hit = true;
-        }
-        if (grp >= 0) K[grp] = (unsigned)min((long long)have, sq);
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const unsigned need = !hit && K[i] > 0 && K[i] < cnt[i] ? K[i] : 0u;
-        // the warp whose bins hold the need-th key
-        if (need > before[i] && need <= before[i] + s.wsum[i][wid]) {
-            unsigned run = before[i] + warp_inclusive_scan(own[i]) - own[i];
-            if (need > run && need <= run + own[i]) {
-                const unsigned q[kPer] = {c[i].w, c[i].z, c[i].y, c[i].x};
-                int k = 0;
-#pragma unroll
-                for (; k < kPer - 1; ++k) {
-                    if (need <= run + q[k]) break;
-                    run += q[k];
-                }
-                s.bin[i] = (unsigned)(b0 + kPer - 1 - k);
-                s.above[i] = run;
-            }
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 || threadIdx.x == 32) {
-        const int i = threadIdx.x ? 1 : 0;
-        const unsigned Ki = i ? K[1] : K[0], ci = i ? cnt[1] : cnt[0];
-        SelGroup &G = st->g[i];
-        G.cnt = ci;
-        G.K = Ki;
-        const int b = (int)s.bin[i];
-        if (hit && i == heavy) {
-            G.mode = 2;
-            G.thr = gkey(s.guess);
-            G.take_eq = (unsigned)(sq - (long long)ci);
-        } else if (Ki == 0) {
-            G.mode = 0;
-        } else if (Ki >= ci) {
-            G.mode = 1;
-        } else if (b > 0 && b < kHistBins - 1) {
-            G.mode = 2;
-            G.thr = gkey(b + kClampLo);
-            G.take_eq = Ki - s.above[i];
-        } else {
-            // the threshold lies in a clamped end bucket: exact radix select over its keys
-            G.mode = 3;
-            G.need = Ki - s.above[i];
-            G.base = b == kHistBins - 1 ? gkey(kHistBins - 1 + kClampLo) : 0u;
-            G.top = b == kHistBins - 1 ? 1ull << 32 : (unsigned long long)gkey(kClampLo) + 1ull;
-            const unsigned long long range = G.top - G.base;
-            const unsigned bits = range > 1 ? 64 - __clzll(range - 1ull) : 0;
-            G.shift = bits > kHistBits ? bits - kHistBits : 0;
-            s.slow = 1;
-        }
-        if (i == 0) s.base = hit;
-    }
-    __syncthreads();
-    return true;
-}
-
 // The ties of group i among the window's bits (first node w0) whose rank by id, `done` of them in the
 // windows before, is below `take`.  All threads.
-__device__ __noinline__ void take_ties(const Ctx x, int kind, int w0, int words, int i, unsigned take, unsigned &done,
-                          unsigned long long &inc, unsigned long long &weight) {
+__device__ __noinline__ unsigned take_ties(int kind, int w0, int words, int i, unsigned take, unsigned done) {
     Shared &s = sh();
     const int tie_gain = (int)(s.st.g[i].thr ^ 0x80000000u);
     const int per = (words + kT - 1) / kT, q0 = (int)threadIdx.x * per, q1 = min(q0 + per, words);
     unsigned own = 0;
+#pragma unroll 1
     for (int q = q0; q < q1; ++q) own += (unsigned)__popc(s.bits[i][q]);
-    unsigned long long tot;
-    const unsigned run = (unsigned)block_exclusive_scan<unsigned long long>((unsigned long long)own, s.red, &tot);
-    const unsigned want = min(take - done, (unsigned)tot);  // this window's first `want` ties
+    unsigned tot;
+    const unsigned run = block_scan32<kT>(own, s.red, &tot);
+    const unsigned want = min(take - done, tot);  // this window's first `want` ties
+#pragma unroll 1
     for (unsigned c0 = 0; c0 < want; c0 += kStep) {
         // a tie's rank is its place in the list
         const unsigned c1 = min(c0 + (unsigned)kStep, want), at = s.nchosen;
         if (run < c1 && run + own > c0) {
             unsigned rank = run;
+#pragma unroll 1
             for (int q = q0; q < q1; ++q) {
                 unsigned bits = s.bits[i][q];
                 while (bits) {
@@ -417,35 +371,99 @@ __device__ __noinline__ void take_ties(const Ctx x, int kind, int w0, int words,
         __syncthreads();
         if (threadIdx.x == 0) s.nchosen = at + (c1 - c0);
         __syncthreads();
-        if (s.nchosen > (unsigned)(kChosenCap - kStep)) flush_chosen(x, kind, inc, weight);
+        if (s.nchosen > (unsigned)(kChosenCap - kStep)) flush_chosen(kind);
         __syncthreads();
     }
-    done += (unsigned)tot;
+    return done + tot;
 }
 
 // Sum over the blocks [0, n) of their tie counts of group i (one load per lane, all lanes get it).
-__device__ __forceinline__ unsigned sum_ties(const Ctx &x, int n, int i) {
+__device__ __forceinline__ unsigned sum_ties(int n, int i) {
     const int lane = threadIdx.x & 31;
-    return __reduce_add_sync(0xffffffffu, lane < n ? __ldcg(&x.rd()->ties[lane][i]) : 0u);
+    return __reduce_add_sync(0xffffffffu, lane < n ? __ldcg(&global_round()->ties[lane][i]) : 0u);
+}
+
+// The application when a block's candidates did not fit its list: its nodes read again.  ties: the block's
+// ties met are added to ntie, and marked when the range is one window.
+__device__ __noinline__ void apply_nodes(int kind, int floor, bool one_win) {
+    Shared &s = sh();
+    const Ctx &x = s.x;
+    const Taken d = s.taken;
+    const Filter f = filter(kind, &s.st, floor);
+    unsigned n0 = 0, n1 = 0;
+    visit_nodes(x.lo, x.hi, f.floor, kind == SEL_REBAL, s.a.m.side, [&](const Step &t) {
+        unsigned in = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int grp = t.side(q);
+            const int what = f.in(t, q) ? d(grp, t.g[q]) : 0;
+            if (what == 2) in |= 1u << q;
+            if (what == 1) {
+                if (one_win) atomicOr(&s.bits[grp][(t.node(q) - x.lo) >> 5], 1u << ((t.node(q) - x.lo) & 31));
+                if (grp) ++n1;
+                else ++n0;
+            }
+        }
+        __syncwarp();
+        unsigned o = warp_places(&s.nchosen, (unsigned)__popc(in));
+        if (in)
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (in >> q & 1u) choose(kind, o++, t.node(q), t.side(q), t.g[q]);
+        __syncthreads();
+        if (s.nchosen > (unsigned)(kChosenCap - kStep)) flush_chosen(kind);
+        __syncthreads();
+    });
+    n0 = __reduce_add_sync(0xffffffffu, n0);
+    n1 = __reduce_add_sync(0xffffffffu, n1);
+    if ((threadIdx.x & 31) == 0 && n0) atomicAdd(&s.ntie[0], n0);
+    if ((threadIdx.x & 31) == 0 && n1) atomicAdd(&s.ntie[1], n1);
+}
+
+// The first `take` ties of group i of a range longer than the bitmap: window by window, the bitmap filled from
+// the nodes again, by the sides before this selection (nodes of the other group may have flipped; rebalance
+// sides have not changed).
+__device__ __noinline__ void take_windows(int kind, int i, unsigned take) {
+    Shared &s = sh();
+    const Ctx &x = s.x;
+    const int thr = (int)(s.st.g[i].thr ^ 0x80000000u);
+    Filter f = filter(kind, &s.st, thr);
+    f.side = i;
+    unsigned done = 0;
+    for (int w0 = x.lo; w0 < x.hi && done < take; w0 += kWin) {
+        __syncthreads();
+        for (int q = threadIdx.x; q < kWinWords; q += kT) s.bits[i][q] = 0;
+        __syncthreads();
+        visit_nodes(w0, min(x.hi, w0 + kWin), thr, kind == SEL_REBAL, kind == SEL_REBAL ? s.a.m.side : s.a.m.prev,
+                    [&](const Step &t) {
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            if (t.g[q] == thr && f.in(t, q))
+                                atomicOr(&s.bits[i][(t.node(q) - w0) >> 5], 1u << ((t.node(q) - w0) & 31));
+                    });
+        __syncthreads();
+        done = take_ties(kind, w0, kWinWords, i, take, done);
+    }
 }
 
 // The exact radix passes for a threshold in a clamped end bucket (rare).
-__device__ __noinline__ void exact_threshold(const Ctx x, int kind, bool need_w) {
+__device__ __noinline__ void exact_threshold(int kind, bool need_w) {
     Shared &s = sh();
+    const Ctx &x = s.x;
     RState *st = &s.st;
     unsigned *total = &s.a.m.ls->hist[0][0];
     const Filter f = filter(kind, st, INT_MIN);
     for (int pass = 0; pass < 3; ++pass) {
         if (!x.solo) {
-            x.sync();  // every block has read the histogram
+            cluster_sync();  // every block has read the histogram
             if (x.r == 0)
                 for (int i = threadIdx.x; i < 2 * kHistBins; i += kT) total[i] = 0;
-            x.sync();
+            cluster_sync();
         }
         __syncthreads();
         for (int i = threadIdx.x; i < 2 * kHistBins; i += kT) (&st->hist[0][0])[i] = 0;
         __syncthreads();
-        visit_nodes(x, x.lo, x.hi, f.floor, need_w, s.a.m.side, [&](const Step &t) {
+        visit_nodes(x.lo, x.hi, f.floor, need_w, s.a.m.side, [&](const Step &t) {
 #pragma unroll 1
             for (int i = 0; i < 2; ++i) {
                 const SelGroup &G = st->g[i];
@@ -459,7 +477,7 @@ __device__ __noinline__ void exact_threshold(const Ctx x, int kind, bool need_w)
                 }
             }
         });
-        sum_hist(x);
+        sum_hist();
         d_sel_find_exact(st, s.a.status, st->hist);
         __syncthreads();
     }
@@ -472,8 +490,9 @@ __device__ __noinline__ void exact_threshold(const Ctx x, int kind, bool need_w)
 // for the application, which otherwise reads the nodes again.  Rebalance rounds after a level's first
 // start from the last round's threshold gain: nodes below it are not looked at, those at it go
 // straight into the tie bitmap, and only when too few are left does the pass start over.
-__device__ __noinline__ void select_nodes(const Ctx x, int kind) {
+__device__ __noinline__ void select_nodes(int kind) {
     Shared &s = sh();
+    const Ctx &x = s.x;
     const LoopArgs &a = s.a;
     RState *st = &s.st;
     const int lo = x.lo, hi = x.hi;
@@ -486,7 +505,7 @@ __device__ __noinline__ void select_nodes(const Ctx x, int kind) {
         const Filter f = filter(kind, st, kind == SEL_REFINE ? 0 : (guess ? gv : INT_MIN));
         clear_pass(one_win ? words : 0);
         unsigned mine = 0;  // ties met
-        visit_nodes(x, lo, hi, f.floor, need_w, a.m.side, [&](const Step &t) {
+        visit_nodes(lo, hi, f.floor, need_w, a.m.side, [&](const Step &t) {
             unsigned cand = 0, at = 0;
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
@@ -509,13 +528,14 @@ __device__ __noinline__ void select_nodes(const Ctx x, int kind) {
             }
             if (__any_sync(0xffffffffu, *(volatile unsigned *)&s.nlist <= (unsigned)kListCap)) {
                 unsigned o = warp_places(&s.nlist, (unsigned)__popc(cand));
+                if (cand)
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (cand >> q & 1u) {
-                        if (o < (unsigned)kListCap)
-                            s.list[o] = make_int2(t.node(q) | (int)((unsigned)(f.side < 0 ? t.side(q) : f.side) << 31), t.g[q]);
-                        ++o;
-                    }
+                    for (int q = 0; q < 8; ++q)
+                        if (cand >> q & 1u) {
+                            if (o < (unsigned)kListCap)
+                                s.list[o] = make_int2(t.node(q) | (int)((unsigned)(f.side < 0 ? t.side(q) : f.side) << 31), t.g[q]);
+                            ++o;
+                        }
             }
         });
         unsigned ties = 0;
@@ -523,148 +543,99 @@ __device__ __noinline__ void select_nodes(const Ctx x, int kind) {
             mine = __reduce_add_sync(0xffffffffu, mine);
             if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&s.ntie[heavy], mine);
             __syncthreads();
-            if (threadIdx.x == 0 && !x.solo) x.rd()->ties[x.r][heavy] = s.ntie[heavy];
+            if (threadIdx.x == 0 && !x.solo) global_round()->ties[x.r][heavy] = s.ntie[heavy];
         }
-        sum_hist(x);
-        if (guess) ties = x.solo ? s.ntie[heavy] : sum_ties(x, x.C, heavy);
-        if (find_threshold(kind, guess, ties)) break;
+        sum_hist();
+        if (guess) ties = x.solo ? s.ntie[heavy] : sum_ties(x.C, heavy);
+        if (find_threshold<kT>(st, s.find, kind, a.sq, guess, gv, ties)) break;
         guess = false;
         if (!x.solo) {  // start over: the shared histogram is cleared between two barriers
-            x.sync();
+            cluster_sync();
             if (x.r == 0)
                 for (int i = threadIdx.x; i < 2 * kHistBins; i += kT) (&a.m.ls->hist[0][0])[i] = 0;
-            x.sync();
+            cluster_sync();
         }
         __syncthreads();
     }
-    const bool hit = s.base != 0;  // the threshold is the guess: its ties are in the bitmap and counted
-    const bool slow = s.slow != 0;
-    if (slow) exact_threshold(x, kind, need_w);
-    const SelGroup G0 = st->g[0], G1 = st->g[1];
-    // some: a group whose threshold's ties are not all taken (or not counted yet)
-    bool some[2];
+    const bool hit = s.find.hit != 0;  // the threshold is the guess: its ties are in the bitmap and counted
+    const bool slow = s.find.slow != 0;
+    if (slow) exact_threshold(kind, need_w);
+    Taken d;
+    d.hit = hit;
+#pragma unroll
     for (int i = 0; i < 2; ++i) {
-        const SelGroup &G = i ? G1 : G0;
-        some[i] = G.mode == 2;
-        if (some[i] && !slow && !hit) some[i] = st->hist[i][(int)(G.thr ^ 0x80000000u) - kClampLo] > G.take_eq;
+        d.mode[i] = st->g[i].mode;
+        d.thr[i] = st->g[i].thr;
+        d.some[i] = d.mode[i] == 2 &&
+                    (slow || hit || st->hist[i][(int)(d.thr[i] ^ 0x80000000u) - kClampLo] > st->g[i].take_eq);
     }
-    if (threadIdx.x == 0) s.nchosen = 0;
+    if (threadIdx.x == 0) {
+        s.nchosen = 0;
+        s.taken = d;
+    }
     if (guess && !hit) {  // the threshold lies above the guess: its ties come from the list
+#pragma unroll 1
         for (int q = threadIdx.x; q < words; q += kT) s.bits[0][q] = s.bits[1][q] = 0;
         if (threadIdx.x < 2) s.ntie[threadIdx.x] = 0;
     }
     __syncthreads();
-    unsigned long long inc = 0, weight = 0;
-    unsigned t0 = 0, t1 = 0;  // ties this thread met
-    auto taken = [&](int v, int grp, int g) -> bool {  // whether a candidate is taken; ties are marked
-        const SelGroup &G = grp ? G1 : G0;
-        if (G.mode == 1) return true;
-        if (G.mode != 2) return false;
-        const unsigned k = gkey(g);
-        if (k != G.thr || hit) return k > G.thr;
-        if (!(grp ? some[1] : some[0])) return true;
-        if (one_win) atomicOr(&s.bits[grp][(v - lo) >> 5], 1u << ((v - lo) & 31));
-        (grp ? t1 : t0) += 1;
-        return false;
-    };
     if (s.nlist <= (unsigned)kListCap) {
         const int n = (int)s.nlist;
+#pragma unroll 1
         for (int i0 = 0; i0 < n; i0 += kT) {
             const int i = i0 + (int)threadIdx.x;
             const int2 c = i < n ? s.list[i] : make_int2(0, 0);
             const int v = c.x & 0x7fffffff, grp = (int)((unsigned)c.x >> 31);
-            const bool in = i < n && taken(v, grp, c.y);
+            const int what = i < n ? d(grp, c.y) : 0;
+            if (what == 1) {
+                if (one_win) atomicOr(&s.bits[grp][(v - lo) >> 5], 1u << ((v - lo) & 31));
+                atomicAdd(&s.ntie[grp], 1u);
+            }
             __syncwarp();
-            const unsigned o = warp_places(&s.nchosen, in);
-            if (in) choose(kind, o, v, grp, c.y);
+            const unsigned o = warp_places(&s.nchosen, what == 2);
+            if (what == 2) choose(kind, o, v, grp, c.y);
         }
     } else {
-        const Filter f = filter(kind, st, kind == SEL_REFINE ? 0 : (guess ? gv + 1 : INT_MIN));
-        visit_nodes(x, lo, hi, f.floor, need_w, a.m.side, [&](const Step &t) {
-            unsigned in = 0;
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (f.in(t, q) && taken(t.node(q), f.side < 0 ? t.side(q) : f.side, t.g[q])) in |= 1u << q;
-            __syncwarp();
-            unsigned o = warp_places(&s.nchosen, (unsigned)__popc(in));
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (in >> q & 1u) choose(kind, o++, t.node(q), f.side < 0 ? t.side(q) : f.side, t.g[q]);
-            __syncthreads();
-            if (s.nchosen > (unsigned)(kChosenCap - kStep)) flush_chosen(x, kind, inc, weight);
-            __syncthreads();
-        });
+        apply_nodes(kind, kind == SEL_REFINE ? 0 : (guess ? gv + 1 : INT_MIN), one_win);
     }
-    if (some[0] || some[1]) {  // the same in every block
-        unsigned take[2] = {0, 0};
-        if (!hit) {
-            t0 = __reduce_add_sync(0xffffffffu, t0);
-            t1 = __reduce_add_sync(0xffffffffu, t1);
-            if ((threadIdx.x & 31) == 0 && t0) atomicAdd(&s.ntie[0], t0);
-            if ((threadIdx.x & 31) == 0 && t1) atomicAdd(&s.ntie[1], t1);
-        }
+    if (d.some[0] || d.some[1]) {  // the same in every block
         __syncthreads();
         if (!x.solo && !hit) {
-            if (threadIdx.x < 2) x.rd()->ties[x.r][threadIdx.x] = s.ntie[threadIdx.x];
-            x.sync();
+            if (threadIdx.x < 2) global_round()->ties[x.r][threadIdx.x] = s.ntie[threadIdx.x];
+            cluster_sync();
         }
-        // ties are taken by ascending id: the blocks before this one take theirs first
+#pragma unroll 1
         for (int i = 0; i < 2; ++i) {
-            if (!some[i]) continue;
-            const unsigned want = (i ? G1 : G0).take_eq;
-            const unsigned before = x.solo ? 0u : sum_ties(x, x.r, i);
-            take[i] = before >= want ? 0u : min(s.ntie[i], want - before);
-        }
-        for (int i = 0; i < 2; ++i) {
-            if (take[i] == 0) continue;  // block-uniform
-            unsigned done = 0;
-            if (one_win) {
-                take_ties(x, kind, lo, words, i, take[i], done, inc, weight);
-                continue;
-            }
-            // windows of the range: the bitmap is filled from the nodes again, by the sides before this
-            // selection (nodes of the other group may have flipped); rebalance sides have not changed
-            const int thr = (int)((i ? G1 : G0).thr ^ 0x80000000u);
-            Filter f = filter(kind, st, thr);
-            f.side = i;
-            for (int w0 = lo; w0 < hi && done < take[i]; w0 += kWin) {
-                __syncthreads();
-                for (int q = threadIdx.x; q < kWinWords; q += kT) s.bits[i][q] = 0;
-                __syncthreads();
-                visit_nodes(x, w0, min(hi, w0 + kWin), thr, need_w, kind == SEL_REBAL ? a.m.side : a.m.prev,
-                            [&](const Step &t) {
-#pragma unroll
-                                for (int q = 0; q < 8; ++q)
-                                    if (t.g[q] == thr && f.in(t, q))
-                                        atomicOr(&s.bits[i][(t.node(q) - w0) >> 5], 1u << ((t.node(q) - w0) & 31));
-                            });
-                __syncthreads();
-                take_ties(x, kind, w0, kWinWords, i, take[i], done, inc, weight);
-            }
+            if (!(i ? d.some[1] : d.some[0])) continue;
+            // ties are taken by ascending id: the blocks before this one take theirs first
+            const unsigned want = st->g[i].take_eq, before = x.solo ? 0u : sum_ties(x.r, i);
+            const unsigned take = before >= want ? 0u : min(s.ntie[i], want - before);
+            if (take == 0) continue;  // block-uniform
+            if (one_win) take_ties(kind, lo, words, i, take, 0);
+            else take_windows(kind, i, take);
         }
     }
-    flush_chosen(x, kind, inc, weight);
+    flush_chosen(kind);
     if (threadIdx.x == 0) {
-        const SelGroup &G = heavy > 0 ? G1 : G0;
-        s.guessed = kind == SEL_REBAL && heavy >= 0 && !slow && G.mode == 2;
-        s.guess = (int)(G.thr ^ 0x80000000u);
+        const int i = heavy > 0;
+        s.guessed = kind == SEL_REBAL && heavy >= 0 && !slow && d.mode[i] == 2;
+        s.guess = (int)((i ? d.thr[1] : d.thr[0]) ^ 0x80000000u);
     }
-    inc = warp_sum(inc);
-    weight = warp_sum(weight);
-    if ((threadIdx.x & 31) == 0 && inc) atomicAdd(&x.rd()->inc, inc);
-    if ((threadIdx.x & 31) == 0 && weight) atomicAdd(&x.rd()->weight, weight);
-    x.sel_sync();
+    if (kind != SEL_REBAL && threadIdx.x == 0) add_sums();
+    sel_sync();
 }
 
 // The level's sides, pairs and gains (what k_level_start, k_hedge_n1 and k_node_gain do on large levels), by
 // all blocks, hyperedge by hyperedge: its side-1 pins counted, its pair stored, its contributions added to
 // its pins' gains.  Up to 32 pins take one thread, more a warp.  Levels whose nodes have many incidences add
 // up in shared memory first: few nodes would take many atomics each.
-__device__ __noinline__ void start_level(const Ctx x) {
+__device__ __noinline__ void start_level() {
     Shared &s = sh();
+    const Ctx &x = s.x;
     const LoopArgs &a = s.a;
     const MoveArgs &m = a.m;
     const int rank = x.r * kT + (int)threadIdx.x, size = x.C * kT, lane = threadIdx.x & 31;
+#pragma unroll 1
     for (int v = rank; v < m.N; v += size) {
         const uint8_t sd = a.cmap ? __ldg(a.coarse + __ldg(a.cmap + v)) : (uint8_t)1;
         m.side[v] = sd;
@@ -672,15 +643,19 @@ __device__ __noinline__ void start_level(const Ctx x) {
         m.gain[v] = 0;
     }
     if (x.r == x.C - 1)
-        for (int i = threadIdx.x; i < (int)(offsetof(LoopState, w1) / sizeof(unsigned)); i += kT)
+        for (int i = threadIdx.x; i < (int)(offsetof(LoopState, cmd) / sizeof(unsigned)); i += kT)
             reinterpret_cast<unsigned *>(m.ls)[i] = 0;
     constexpr int kAcc = (int)(sizeof(s.chosen) / sizeof(int));
-    int *acc = reinterpret_cast<int *>(s.chosen);
+    int *acc = reinterpret_cast<int *>(sh().chosen);
     const bool priv = m.N <= kAcc && m.P > 8 * m.N;
     if (priv)
         for (int v = threadIdx.x; v < m.N; v += kT) acc[v] = 0;
-    x.sync();
-    auto add = [&](int v, int c) { atomicAdd((priv ? acc : m.gain) + v, c); };
+    cluster_sync();
+    auto add = [&](int v, int c) {
+        if (priv) atomicAdd(acc + v, c);
+        else atomicAdd(m.gain + v, c);
+    };
+#pragma unroll 1
     for (int e0 = (rank & ~31); e0 < m.E; e0 += size) {
         const int e = e0 + lane;
         int b = 0, d = 0;
@@ -696,6 +671,7 @@ __device__ __noinline__ void start_level(const Ctx x) {
             m.pair[e] = (unsigned long long)(unsigned)n0 << 32 | (unsigned)n1;
             const int c0 = w * contrib(n0, n1), c1 = w * contrib(n1, n0);
             if (c0 | c1)
+#pragma unroll 1
                 for (int i = 0; i < d; ++i) {
                     const int c = on1 >> i & 1u ? c1 : c0;
                     if (c) add(__ldg(m.pins + b + i), c);
@@ -714,6 +690,7 @@ __device__ __noinline__ void start_level(const Ctx x) {
             if (lane == 0) m.pair[we] = (unsigned long long)(unsigned)n0 << 32 | (unsigned)n1;
             const int c0 = w * contrib(n0, n1), c1 = w * contrib(n1, n0);
             if (c0 | c1)
+#pragma unroll 1
                 for (int i = lane; i < wd; i += 32) {
                     const int v = __ldg(m.pins + wb + i);
                     const int c = __ldcg(m.side + v) ? c1 : c0;
@@ -726,14 +703,15 @@ __device__ __noinline__ void start_level(const Ctx x) {
         for (int v = threadIdx.x; v < m.N; v += kT)
             if (acc[v]) atomicAdd(m.gain + v, acc[v]);
     }
-    x.sync();
+    cluster_sync();
 }
 
 // Gains after the last selection's moves, by all blocks.  own: exact for the moved nodes too (a
 // rebalance leaves them out: they are on the light side, which stays the light side until the
 // level is done).
-__device__ __noinline__ void update_gains(const Ctx x, bool own) {
+__device__ __noinline__ void update_gains(bool own) {
     Shared &s = sh();
+    const Ctx &x = s.x;
     const MoveArgs &m = s.a.m;
     LoopState *ls = m.ls;
     const uint8_t *wside = own ? m.prev : m.side;
@@ -759,7 +737,7 @@ __device__ __noinline__ void update_gains(const Ctx x, bool own) {
             ls->rd[0].items = 0;
             ls->cmd = 1u | (unsigned)own << 1;
         }
-        x.sync();  // the helpers read the command after this barrier
+        cluster_sync();  // the helpers read the command after this barrier
     } else {
         n = __ldcg(&ls->rd[x.p].ents);
     }
@@ -773,11 +751,11 @@ __device__ __noinline__ void update_gains(const Ctx x, bool own) {
     // a warp per entry, the blocks' first warps first: a short list spreads over all SMs
     const int warp = (tid >> 5) * x.C + x.r, warps = x.C * kWarps;
     move_pass1(m, n, &rd->items, warp, warps, wside, false);
-    x.sync();
+    cluster_sync();
     const unsigned items = __ldcg(&rd->items);
     if (own || items > 0) {
         move_pass2(m, n, items, warp, warps, wside, own);
-        x.sync();
+        cluster_sync();
     }
     if (x.solo) {
         if (x.r != 0) return;
@@ -789,114 +767,42 @@ __device__ __noinline__ void update_gains(const Ctx x, bool own) {
     }
 }
 
-// Sorts keys[0, S) ascending (S a power of two): in registers with warp shuffles where a thread holds
-// one key, in shared memory above.
-__device__ __noinline__ void sort_keys(unsigned long long *keys, int S) {
-    const int t = threadIdx.x;
-    if (S <= kT) {
-        unsigned long long k0 = t < S ? keys[t] : ~0ull;
-        for (int k = 2; k <= S; k <<= 1) {
-            const bool up = (t & k) == 0;
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                unsigned long long o;
-                if (j >= 32) {
-                    __syncthreads();
-                    if (t < S) keys[t] = k0;
-                    __syncthreads();
-                    o = t < S ? keys[t ^ j] : ~0ull;
-                } else {
-                    o = __shfl_xor_sync(0xffffffffu, k0, j);
-                }
-                const bool lower = (t & j) == 0;
-                k0 = (lower == up) == (o < k0) ? o : k0;
-            }
-        }
-        __syncthreads();
-        if (t < S) keys[t] = k0;
-        __syncthreads();
-        return;
-    }
-    for (int k = 2; k <= S; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = t; i < S; i += kT) {
-                const int q = i ^ j;
-                if (q > i) {
-                    const unsigned long long u = keys[i], v = keys[q];
-                    if ((u > v) == ((i & k) == 0)) { keys[i] = v; keys[q] = u; }
-                }
-            }
-            __syncthreads();
-        }
-}
-
 // Ordered move of the rebalance (reading C13), alike in every selecting block; block r moves every
-// C-th node.  The shortest prefix by (gain descending, id ascending) whose weight reaches `need`: when
-// all candidates together do not reach it (most rounds) they all move and need no order.
-__device__ __noinline__ void rebal_move(const Ctx x) {
+// C-th node of the prefix.
+__device__ __noinline__ void rebal_move() {
     Shared &s = sh();
+    const Ctx &x = s.x;
     const LoopArgs &a = s.a;
     unsigned long long *keys = s.keys();
     RState *st = &s.st;
-    const int n = x.solo ? (int)s.nchosen : (int)__ldcg(&x.rd()->cands);
+    const int n = x.solo ? (int)s.nchosen : (int)__ldcg(&global_round()->cands);
     if (n == 0) {
         __syncthreads();
         if (threadIdx.x == 0) st->warn = 1;
-        x.sel_sync();
+        sel_sync();
         return;
     }
-    const long long room = st->room, need = st->need;
     const int heavy = st->heavy;
     int S = 1;
     while (S < n) S <<= 1;
-    long long loc = 0;
+    unsigned total = 0;
+#pragma unroll 1
     for (int i = threadIdx.x; i < S; i += kT) {
         unsigned long long k = ~0ull;
         if (i < n) {
             k = x.solo ? (unsigned long long)~gkey(s.chosen[i].y) << 32 | (unsigned)s.chosen[i].x : __ldcg(a.cand + i);
-            loc += __ldg(a.m.nw + (unsigned)k);
+            total += (unsigned)__ldg(a.m.nw + (unsigned)k);
         }
         keys[i] = k;
     }
-    long long moved = block_sum<long long>(loc, reinterpret_cast<long long *>(s.red));
-    int cut = (int)min((long long)n, a.sq);
-    if (moved >= need || moved > room) {
-        if (threadIdx.x == 0) s.cut = cut;
-        __syncthreads();
-        sort_keys(keys, S);
-        // every thread a run of consecutive nodes; the first node past room, or the first to reach need,
-        // ends the prefix, and its thread knows the weight before or up to it
-        const int per = (n + kT - 1) / kT, i0 = (int)threadIdx.x * per;
-        loc = 0;
-        for (int q = 0; q < per && i0 + q < n; ++q) loc += __ldg(a.m.nw + (unsigned)keys[i0 + q]);
-        long long tot;
-        long long run = block_exclusive_scan<long long>(loc, reinterpret_cast<long long *>(s.red), &tot);
-        long long at = tot;
-        int mine = cut;
-        for (int q = 0; q < per && i0 + q < n; ++q) {
-            const long long w = __ldg(a.m.nw + (unsigned)keys[i0 + q]);
-            if (run + w > room || run + w >= need) {
-                const bool over = run + w > room;  // node i0 + q would exceed room: it stays
-                mine = i0 + q + !over;
-                at = over ? run : run + w;
-                atomicMin(&s.cut, mine);
-                break;
-            }
-            run += w;
-        }
-        __syncthreads();
-        cut = s.cut;
-        if (threadIdx.x == 0) s.moved = tot;
-        __syncthreads();
-        if (mine == cut && at != tot) s.moved = at;
-        __syncthreads();
-        moved = s.moved;
-    }
+    total = block_sum32<kT>(total, s.red);
+    unsigned moved;
+    const int cut = rebal_prefix<kT>(keys, n, a.sq, st->room, st->need, a.m.nw, total, s.red, s.cut, &moved);
     if (threadIdx.x == 0) {
-        st->W[1 - heavy] += (unsigned long long)moved;
-        st->W[heavy] -= (unsigned long long)moved;
+        st->W[1 - heavy] += moved;
+        st->W[heavy] -= moved;
     }
     __syncthreads();
-    unsigned long long inc = 0, weight = 0;
     const int D = x.solo ? 1 : x.C, r = x.solo ? 0 : x.r;
     for (int b0 = 0; b0 < cut; b0 += kStep * D) {
         const int left = min(cut - b0 - r + D - 1, kStep * D) / D;  // this block's nodes of the step
@@ -906,43 +812,28 @@ __device__ __noinline__ void rebal_move(const Ctx x) {
             s.chosen[i] = make_int2(v, 1 - heavy);
         }
         if (threadIdx.x == 0) s.nchosen = (unsigned)max(left, 0);
-        flush_chosen(x, SEL_REFINE, inc, weight);
+        flush_chosen(SEL_REFINE);
     }
-    inc = warp_sum(inc);
-    if ((threadIdx.x & 31) == 0 && inc) atomicAdd(&x.rd()->inc, inc);
-    x.sel_sync();
+    if (threadIdx.x == 0) add_sums();
+    sel_sync();
 }
 
-// The side weights, from side 1's.
-__device__ __noinline__ void sum_weights(const Ctx x) {
-    Shared &s = sh();
-    const MoveArgs &m = s.a.m;
-    unsigned long long w = 0;
-    visit_nodes(x, x.lo, x.hi, INT_MIN, true, m.side, [&](const Step &t) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) w += t.side(q) ? (unsigned)t.w[q] : 0u;
-    });
-    w = block_sum(w, s.red);
-    if (!x.solo) {
-        if (threadIdx.x == 0) m.ls->w1[x.r] = w;
-        x.sync();
-        const int lane = threadIdx.x & 31;
-        w = warp_sum(lane < x.C ? __ldcg(&m.ls->w1[lane]) : 0ull);
-    }
-    if (threadIdx.x == 0) {
-        s.st.W[1] = w;
-        s.st.W[0] = (unsigned long long)s.a.W - w;
-    }
-    __syncthreads();
+// The side weights after a selection's moves (one thread).
+__device__ __forceinline__ void move_weight() {
+    RState &st = sh().st;
+    const unsigned long long w = round_count(&LoopRound::weight);
+    st.W[1] += w;
+    st.W[0] -= w;
 }
 
-__device__ __forceinline__ bool too_large(const Ctx &x) {
-    return sh().a.suspend && x.count(&LoopRound::inc) > (unsigned long long)kLoopMoveInc;
+__device__ __forceinline__ bool too_large() {
+    return sh().a.suspend && round_count(&LoopRound::inc) > (unsigned long long)kLoopMoveInc;
 }
 
 // End of the launch for the selecting blocks (solo: the helpers are sent home).
-__device__ void leave(const Ctx &x, unsigned pending, int it, bool rebal) {
+__device__ __noinline__ void leave(unsigned pending, int it, bool rebal) {
     const LoopArgs &a = sh().a;
+    const Ctx &x = sh().x;
     LoopState *ls = a.m.ls;
     if (x.r == 0 && threadIdx.x == 0) {
         const RState &st = sh().st;
@@ -964,130 +855,127 @@ __device__ void leave(const Ctx &x, unsigned pending, int it, bool rebal) {
         ls->need = st.need;
         if (a.pending_slot) *a.pending_slot = pending;
     }
-    if (x.solo && x.C > 1) x.sync();
+    if (x.solo && x.C > 1) cluster_sync();
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(kLoopThreads, 1) k_refine_loop(const __grid_constant__ LoopArgs a) {
+__global__ void __launch_bounds__(kLoopThreads, 1) k_refine_loop(const __grid_constant__ LoopArgs args) {
     Shared &s = sh();
     cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
-    LoopState *ls = a.m.ls;
-    const int parts = a.solo ? 1 : C;
-    const int R = (int)(((long long)a.m.N + parts - 1) / parts + 31) & ~31;
-    const int lo = a.solo ? 0 : (int)min((long long)R * r, (long long)a.m.N);
-    const int hi = (int)min((long long)lo + R, (long long)a.m.N);
-    Ctx x{r, C, lo, hi, a.solo, false, 1};
-    x.vec = ((reinterpret_cast<uintptr_t>(a.m.gain) | reinterpret_cast<uintptr_t>(a.m.nw)) & 15) == 0 &&
-            ((reinterpret_cast<uintptr_t>(a.m.side) | reinterpret_cast<uintptr_t>(a.m.prev)) & 3) == 0;
     for (int i = threadIdx.x; i < (int)(sizeof(LoopArgs) / sizeof(int)); i += kT)
-        reinterpret_cast<int *>(&s.a)[i] = reinterpret_cast<const int *>(&a)[i];
-    if (threadIdx.x == 0) s.guessed = 0;
+        reinterpret_cast<int *>(&s.a)[i] = reinterpret_cast<const int *>(&args)[i];
     if (threadIdx.x < sizeof(LoopRound) / sizeof(unsigned)) reinterpret_cast<unsigned *>(&s.rd)[threadIdx.x] = 0;
-    __syncthreads();
     RState *st = &s.st;
-    if (a.resume) {
-        x.p = (int)__ldcg(&ls->sel);
-        move_settle(a.m, __ldcg(&ls->rd[x.p].ents), r * kT + (int)threadIdx.x, C * kT);
-        if (a.solo) x.sync();
-    }
-    if (a.start && !a.resume) start_level(x);
-    if (a.solo && r != 0) {  // helper: gain updates as the first block commands
-        for (;;) {
-            x.sync();
-            const unsigned cmd = __ldcg(&ls->cmd);
-            if (cmd == 0) return;
-            x.p = 0;
-            update_gains(x, (cmd & 2u) != 0);
-        }
-    }
+    LoopState *ls = args.m.ls;
     if (threadIdx.x == 0) {
+        const int parts = args.solo ? 1 : C;
+        const int R = (int)(((long long)args.m.N + parts - 1) / parts + 31) & ~31;
+        s.x.r = r;
+        s.x.C = C;
+        s.x.lo = args.solo ? 0 : (int)min((long long)R * r, (long long)args.m.N);
+        s.x.hi = (int)min((long long)s.x.lo + R, (long long)args.m.N);
+        s.x.solo = args.solo;
+        s.x.wvec = (reinterpret_cast<uintptr_t>(args.m.nw) & 15) == 0;
+        s.x.p = args.resume ? (int)__ldcg(&ls->sel) : 1;
+        s.guessed = 0;
+        s.inc = s.weight = 0;
         s.nchosen = 0;
         st->heavy = -1;
         st->warn = 0;
         st->rounds = 0;
         st->slow = 0;
+        st->flag = 0;
         st->room = st->need = 0;
+        // the side weights as the coarser level (or the stop) left them
+        st->W[0] = __ldcg(&ls->W[0]);
+        st->W[1] = __ldcg(&ls->W[1]);
     }
     __syncthreads();
+    const LoopArgs &a = s.a;
+    if (a.resume) {
+        move_settle(a.m, __ldcg(&global_round()->ents), r * kT + (int)threadIdx.x, C * kT);
+        if (a.solo) cluster_sync();
+    }
+    if (a.start && !a.resume) start_level();
+    if (a.solo && r != 0) {  // helper: gain updates as the first block commands
+        if (threadIdx.x == 0) s.x.p = 0;
+        for (;;) {
+            cluster_sync();
+            const unsigned cmd = __ldcg(&ls->cmd);
+            if (cmd == 0) return;
+            update_gains((cmd & 2u) != 0);
+        }
+    }
     int it = 0;
     bool pending = false;   // the last selection's moves are not in the gains yet
     bool in_rebal = false;
+    auto select = [&](int kind) {
+        __syncthreads();
+        if (threadIdx.x == 0) s.x.p ^= 1;
+        __syncthreads();
+        select_nodes(kind);
+        pending = true;
+    };
     if (a.resume) {
         it = (int)__ldcg(&ls->it);
         in_rebal = __ldcg(&ls->rebal) != 0;
         if (threadIdx.x == 0 && in_rebal) {
             st->rounds = __ldcg(&ls->rounds);
             st->heavy = __ldcg(&ls->heavy);
-            st->W[0] = __ldcg(&ls->W[0]);
-            st->W[1] = __ldcg(&ls->W[1]);
             st->room = __ldcg(&ls->room);
             st->need = __ldcg(&ls->need);
             st->flag = 1;
         }
         __syncthreads();
     }
-    if (a.initial && !a.resume) {
-        if (threadIdx.x == 0) {
-            st->W[0] = 0;
-            st->W[1] = (unsigned long long)a.W;
-            d_initial_cond(st, a.max_rounds, a.status, true, a.m0, a.mt);
-        }
-        __syncthreads();
-        while (st->flag) {
-            if (pending) update_gains(x, true);
-            x.p ^= 1;
-            select_nodes(x, SEL_INITIAL);
-            pending = true;
+    // Algorithm 3, then Algorithm 5's iterations, then the rebalance: one loop, so that its phases are one copy
+    // of the code
+    int kind = a.initial && !a.resume ? SEL_INITIAL : (in_rebal ? SEL_REBAL : SEL_REFINE);
+    bool first = !in_rebal;  // the loop condition of this kind is evaluated for the first time
+    bool own = !in_rebal;    // the rebalance's first update covers the refinement's moves, exact for every node
+    if (kind == SEL_INITIAL && threadIdx.x == 0) {
+        st->W[0] = 0;
+        st->W[1] = (unsigned long long)a.W;
+    }
+    for (;;) {
+        // the conditions of the loops: Algorithm 3's share, the iteration count, the balance limit
+        if (!(in_rebal && first == false && kind == SEL_REBAL && st->flag && !pending)) {
             if (threadIdx.x == 0) {
-                const unsigned long long w = x.count(&LoopRound::weight);
-                st->W[0] += w;
-                st->W[1] -= w;
-                d_initial_cond(st, a.max_rounds, a.status, false, a.m0, a.mt);
+                if (kind == SEL_INITIAL) d_initial_cond(st, a.max_rounds, a.status, first, a.m0, a.mt);
+                else if (kind == SEL_REFINE) st->flag = it < a.iters;
+                else d_rebal_cond(st, a.limit0, a.limit1, a.max_rounds, a.status, first);
             }
             __syncthreads();
         }
-    }
-    if (!in_rebal) {
-        while (it < a.iters) {
-            if (pending) update_gains(x, true);
-            x.p ^= 1;
-            select_nodes(x, SEL_REFINE);
-            pending = true;
-            ++it;
-            if (it < a.iters && too_large(x)) {
-                leave(x, 1, it, false);
-                return;
-            }
+        first = false;
+        if (!st->flag) {
+            __syncthreads();
+            if (kind == SEL_REBAL) break;
+            kind = kind == SEL_INITIAL ? SEL_REFINE : SEL_REBAL;
+            first = true;
+            continue;
         }
-        sum_weights(x);
-        if (threadIdx.x == 0) d_rebal_cond(st, a.limit0, a.limit1, a.max_rounds, a.status, true);
-        __syncthreads();
-        if (st->flag && pending && too_large(x)) {
-            leave(x, 1, it, false);
-            return;
-        }
-    }
-    // the first update covers the refinement's moves and has to be exact for every node
-    bool own = !in_rebal;
-    while (st->flag) {
         if (pending) {
-            if (too_large(x)) {
-                leave(x, 1, it, true);
+            if (kind != SEL_INITIAL && too_large()) {
+                leave(1, it, kind == SEL_REBAL && !own);
                 return;
             }
-            update_gains(x, own);
+            update_gains(kind != SEL_REBAL || own);
+            if (kind == SEL_REBAL) own = false;
         }
-        x.p ^= 1;
-        select_nodes(x, SEL_REBAL);
-        rebal_move(x);
-        pending = true;
-        own = false;
-        if (threadIdx.x == 0) d_rebal_cond(st, a.limit0, a.limit1, a.max_rounds, a.status, false);
-        __syncthreads();
+        select(kind);
+        if (kind == SEL_REBAL) {
+            own = false;
+            rebal_move();
+        } else if (threadIdx.x == 0) {
+            move_weight();
+        }
+        if (kind == SEL_REFINE) ++it;
+        in_rebal = false;
     }
-    leave(x, 0, it, false);
+    leave(0, it, false);
 }
 
 // ------------------------------------------------------------------------ host side

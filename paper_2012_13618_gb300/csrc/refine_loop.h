@@ -12,7 +12,7 @@ namespace bp {
 constexpr int kLoopThreads = 512;       // threads per block of the cluster
 constexpr int kLoopMaxCluster = 16;
 constexpr int kMoveRun = 64;            // incidences of a moved node one entry of the move list covers
-constexpr int kItemPins = 512;          // pins of a wide hyperedge one work item covers
+constexpr int kItemPins = 128;          // pins of a wide hyperedge one work item covers (four a lane)
 constexpr int kItemCap = 1 << 16;       // work items a pass may queue (beyond: walked on the spot)
 // Moves of more than this many incidences are brought into the gains by the whole grid instead of
 // the one cluster (levels of more than kLoopAlonePins pins only; smaller ones stay in the cluster).
@@ -30,24 +30,24 @@ constexpr int kMoveFull = 8;
 struct LoopRound {
     unsigned ents, items, cands, pad;
     unsigned long long inc;     // incidences of the moved nodes
-    unsigned long long weight;  // their node weight (initial partition)
+    unsigned long long weight;  // node weight moved to side 1 less that moved to side 0
     unsigned ties[kLoopMaxCluster][2];
 };
 
-// Zero at the start of a level (k_level_start); lives in the handle's small scratch.
+// Lives in the handle's small scratch.  The histogram and the rounds are zero at the start of a level
+// (k_level_start, start_level); the side weights carry over from the coarser level.
 struct LoopState {
     unsigned hist[2][kHistBins];
     LoopRound rd[2];
-    unsigned long long w1[kLoopMaxCluster];  // per-block sums of side 1's weight
     unsigned cmd;      // next step of the helper blocks: 0 leave, else 1 | own << 1
     unsigned pending;  // the launch stopped after a selection too large for one cluster
     unsigned sel;      // which LoopRound the last selection used
     unsigned it;       // refinement iterations done
     unsigned status0;  // the level's rebalance ran out of candidates (the last level written is 0)
+    unsigned long long W[2];  // side weights
     // a stop inside the rebalance: its state
     unsigned rebal, rounds;
     int heavy;
-    unsigned long long W[2];
     long long room, need;
 };
 

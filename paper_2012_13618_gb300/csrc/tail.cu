@@ -21,10 +21,14 @@
 // block on identical data and come out identical in every block: no block waits on another except
 // at a cluster barrier, and every block runs the same sequence of barriers.
 //
-// Gains use the weighted degree D[v] = sum of w_e over v's hyperedges, computed once per level:
-// gain[v] = -D[v] + sum over v's CUT hyperedges of w_e (1 + [v alone on its side]), which is
-// Algorithm 4's sum regrouped (an uncut hyperedge contributes -w_e to every pin, a cut one +w_e to
-// a pin alone on its side); only cut hyperedges then touch the node arrays.
+// Refinement runs in the first block alone, on shared memory: the sides, gains, weights and weighted
+// degrees of a level's nodes, and its pins and hyperedge offsets (16-bit) where they fit.  A round is then a
+// pass over the level's pins at shared-memory latency and a selection with block barriers only;
+// spread over the cluster the same pass spent 29 us on streaming chunks, barriers and gathering slices, and a
+// one-shot bisection of 1,000 nodes 365 of its 476 us there.  Gains use the weighted degree D[v] = sum of w_e
+// over v's hyperedges, computed once per level: gain[v] = -D[v] + sum over v's CUT hyperedges of
+// w_e (1 + [v alone on its side]), which is Algorithm 4's sum regrouped (an uncut hyperedge contributes -w_e to
+// every pin, a cut one +w_e to a pin alone on its side); only cut hyperedges then touch the gains.
 //
 // Results are the same integers as the grid path's: minima and sums are order-independent, ties
 // are broken by ids, and the coarse numbering, the contraction order and the selection follow the
@@ -34,6 +38,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <mutex>
@@ -44,6 +49,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "refine_dev.cuh"
+#include "select_dev.cuh"
 #include "tail.h"
 
 namespace bp {
@@ -55,6 +61,7 @@ namespace {
 constexpr int kTT = kTailThreads;
 constexpr int kNT = kTailNodes;
 constexpr int kQ = kTailChunk;
+constexpr int kThreadPins = 32; // refinement: hyperedges up to this degree: one thread; above: one warp
 constexpr int kThreadDeg = 16;  // hyperedges up to this degree: one thread; above: one warp
 constexpr int kWarpDeg = 256;   // contraction: above this, the whole block (bitmap)
 
@@ -68,12 +75,9 @@ constexpr int kStagePins = 2 * kQ + 4;                       // pins[p0 .. p1) f
 constexpr size_t kStageBytes = 4 * (size_t)(kStageHoff + kStagePins);
 constexpr int kChunkHedges = kQ / 2 + 1;
 
-// Dynamic shared memory: two chunk stages at the start, then one of two views.
-// Coarsening: R0 = 8 kNT bytes (matching keys; later two int arrays), R1 = 4 kNT (matched
+// Dynamic shared memory of the coarsening: two chunk stages at the start, then R0 = 8 kNT bytes (matching keys; later two int arrays), R1 = 4 kNT (matched
 // hyperedges; later coarse ids), BM = kNT bits, SW = kNT / 32 word prefixes, then the
-// contraction's per-chunk counts and lists.  Refinement: partial and final gains, the block's
-// slice of the weighted degrees, two side arrays, the selection groups, the selection state, the
-// rebalance's sort keys and candidate list, and the passes' list of wide hyperedges.
+// contraction's per-chunk counts and lists.  The refinement takes the whole of it again (struct Tiny).
 constexpr size_t kSTG = 0;
 constexpr size_t kV = kSTG + 2 * kStageBytes;
 
@@ -86,21 +90,37 @@ constexpr size_t kCL = kCC + 4 * (size_t)(kChunkHedges + 3);    // chunk: tier /
 constexpr int kCListMax = 3 * (kQ / 9 + 8);                     // >= 3 ints per hyperedge of degree > 8
 constexpr size_t kCoarsenEnd = kCL + 4 * (size_t)kCListMax;
 
-constexpr int kSliceMax = kNT / 4 + 8;                          // a slice has <= ceil(N / 4) nodes
-constexpr size_t kGP = kV;                                      // partial gains
-constexpr size_t kGF = kGP + 4 * (size_t)kNT;                   // final gains
-constexpr size_t kDS = kGF + 4 * (size_t)kNT;                   // weighted degrees of the slice
-constexpr size_t kSA = kDS + 4 * (size_t)kSliceMax;
-constexpr size_t kSB = kSA + (size_t)kNT;
-constexpr size_t kGR = kSB + (size_t)kNT;
-constexpr size_t kST = kGR + (size_t)kNT;
-constexpr size_t kKY = kST + ((sizeof(RState) + 255) & ~size_t(255));
-constexpr int kRebalKeys = 256;  // >= the next power of two of ceil(sqrt(kNT))
-constexpr size_t kLS = kKY + 8 * (size_t)kRebalKeys;
-constexpr size_t kWL = kLS + 4 * (size_t)kRebalKeys;           // wide hyperedges of a chunk
-constexpr size_t kRefineEnd = kWL + 4 * (size_t)(kChunkHedges + 3);
+constexpr int kTieWords = (kNT + 31) / 32;
+constexpr int kRebalKeys = 128;  // >= the next power of two of ceil(sqrt(kNT))
+constexpr size_t kSmemMax = 216 * 1024;  // with the kernel's static arrays (9.6 KB) below the 227 KB of a block
 
-constexpr size_t kSmemBytes = kCoarsenEnd > kRefineEnd ? kCoarsenEnd : kRefineEnd;
+// The level at hand: offsets of its arrays in the block's shared memory, so that every access is known to be
+// a shared one.  Kept in shared memory itself: passed by value it went through each thread's stack, and
+// 512 stacks do not fit the little L1 this launch leaves.
+struct TinyLevel {
+    int N, E, P;
+    const int *hoff, *pins, *hw;
+    int gain, deg, nw, wide, sp, so;  // offsets: gains, weighted degrees, weights; wide hyperedges, 16-bit pins
+    bool staged;                      // and offsets, when the hyperedges are staged
+};
+
+// Shared memory of the refinement: this, then the level's node arrays and its staged hyperedges.
+struct Tiny {
+    alignas(16) RState st;
+    TinyLevel lev;
+    FindScratch find;
+    CutScratch cut;
+    unsigned red[32];
+    unsigned ncand, nwide;
+    int wdelta;                                // weight moved to side 1 less that moved to side 0
+    unsigned long long keys[kRebalKeys];       // the rebalance's candidates: gain descending << 32 | node
+    unsigned tie[2][kTieWords], pre[kTieWords];
+    uint8_t side[2][(kNT + 15) & ~15];
+};
+static_assert(offsetof(RState, hist) % 16 == 0, "the histogram is read in 16-byte pieces");
+constexpr size_t kTinyFixed = (sizeof(Tiny) + 15) & ~size_t(15);
+static_assert(kTinyFixed + 12 * (size_t)kNT <= kSmemMax && kCoarsenEnd <= kSmemMax, "shared memory");
+constexpr size_t kSmemBytes = kSmemMax;
 
 __device__ __forceinline__ void csync() { cg::this_cluster().sync(); }
 
@@ -711,121 +731,367 @@ __device__ bool tail_coarsen(const TailArgs &a, const TLev &f, TLev &c, size_t *
 }
 
 // ------------------------------------------------------------------------------ refinement
-// A pass of per-hyperedge contributions into the partial array gp, then the reduce-scatter: the
-// block's slice gets the sum over all blocks (minus the slice's weighted degrees when ds_sub);
-// with `all`, every block then gathers the other slices.
-struct Refine {
-    int *gp, *gf, *ds, *wl, *cnt;
+// One block, a level in shared memory.  Level data that other blocks wrote in this launch is read through L2.
+// Loops are unrolled sparingly (select_dev.cuh says why).
+__device__ __forceinline__ char *tiny_at(int off) {
+    extern __shared__ __align__(16) char tail_smem[];
+    return tail_smem + off;
+}
+__device__ __forceinline__ Tiny &tiny() { return *reinterpret_cast<Tiny *>(tiny_at(0)); }
+__device__ __forceinline__ int *tiny_ints(int off) { return reinterpret_cast<int *>(tiny_at(off)); }
+
+// Pins of the level: staged in shared memory, or in global memory.
+struct StagedPins {
+    const uint16_t *p;
+    __device__ __forceinline__ int operator()(int i) const { return (int)p[i]; }
+};
+struct GlobalPins {
+    const int *p;
+    __device__ __forceinline__ int operator()(int i) const { return __ldcg(p + i); }
 };
 
-template <class One, class Wide>
-__device__ void refine_pass(const TailArgs &a, const TLev &L, const Chunks &ch, char *smem,
-                            const Refine &R, int *out, bool sub_ds, bool all, int lv, One one,
-                            Wide wide) {
-    cg::cluster_group cl = cg::this_cluster();
-    const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
-    const int N = L.N;
-    trace(a, lv, 20);
-    for (int v = threadIdx.x; v < N; v += kTT) R.gp[v] = 0;
-    __syncthreads();
-    stream(L, ch, smem, [&](const Win &w) { win_hedges(w, R.wl, R.cnt, [&](int e, int b, int d) { one(w, e, b, d); },
-                                                       [&](int e, int b, int d) { wide(w, e, b, d); }); });
-    trace(a, lv, 21);
-    csync();
-    trace(a, lv, 22);
-    const int nlo = slice_lo(N, r, C), nhi = slice_lo(N, r + 1, C);
-    for (int v = nlo + (int)threadIdx.x; v < nhi; v += kTT) {
-        int x[kTailMaxCluster];
-#pragma unroll
-        for (int q = 0; q < kTailMaxCluster; ++q) x[q] = q < C ? remote(R.gp, q)[v] : 0;
-        int s = 0;
-#pragma unroll
-        for (int q = 0; q < kTailMaxCluster; ++q) s += x[q];
-        out[v - (all ? 0 : nlo)] = sub_ds ? s - R.ds[v - nlo] : s;
+// Node arrays and, where they fit, the hyperedges of L into shared memory.
+__device__ __noinline__ void tiny_load(const TLev &L) {
+    Tiny &s = tiny();
+    const int n4 = 4 * ((L.N + 3) & ~3);
+    const int wide_cap = L.P / (kThreadPins + 1) + 1;
+    TinyLevel t;
+    t.N = L.N; t.E = L.E; t.P = L.P;
+    t.hoff = L.hoff; t.pins = L.pins; t.hw = L.hw;
+    t.gain = (int)kTinyFixed;
+    t.deg = t.gain + n4;
+    t.nw = t.deg + n4;
+    t.wide = t.nw + n4;
+    t.sp = (t.wide + 4 * wide_cap + 7) & ~7;
+    t.so = t.sp + 2 * ((L.P + 3) & ~3);
+    t.staged = L.P < 65536 && kTinyFixed + 3 * (size_t)n4 + 4 * (size_t)wide_cap + 16 + 2 * (size_t)L.P + 2 * (size_t)L.E <= kSmemMax;
+    if (threadIdx.x == 0) {
+        s.lev = t;
+        s.nwide = 0;
     }
-    csync();
-    trace(a, lv, 23);
-    if (all) {
-        // the other blocks' slices, eight loads in flight per thread
-        for (int v0 = threadIdx.x; v0 < N; v0 += 8 * kTT) {
-            int x[8];
+    __syncthreads();
+#pragma unroll 1
+    for (int v = threadIdx.x; v < L.N; v += kTT) {
+        tiny_ints(t.nw)[v] = __ldcg(L.nw + v);
+        tiny_ints(t.deg)[v] = 0;
+    }
+    if (t.staged) {
+        uint16_t *sp = reinterpret_cast<uint16_t *>(tiny_at(t.sp)), *so = reinterpret_cast<uint16_t *>(tiny_at(t.so));
+        const bool vec = (reinterpret_cast<uintptr_t>(L.pins) & 15) == 0;
+        const int quads = vec ? L.P >> 2 : 0;
+#pragma unroll 1
+        for (int i0 = threadIdx.x; i0 < quads; i0 += 4 * kTT) {
+            int4 x[4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int v = v0 + k * kTT;
-                x[k] = 0;
-                if (v < N && (v < nlo || v >= nhi)) x[k] = remote(out, slice_of(N, v, C))[v];
+            for (int k = 0; k < 4; ++k)
+                if (i0 + k * kTT < quads) x[k] = __ldcg(reinterpret_cast<const int4 *>(L.pins) + i0 + k * kTT);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (i0 + k * kTT < quads)
+                    *reinterpret_cast<uint2 *>(sp + 4 * (i0 + k * kTT)) =
+                        make_uint2((unsigned)x[k].x | (unsigned)x[k].y << 16, (unsigned)x[k].z | (unsigned)x[k].w << 16);
+        }
+#pragma unroll 1
+        for (int i = 4 * quads + (int)threadIdx.x; i < L.P; i += kTT) sp[i] = (uint16_t)__ldcg(L.pins + i);
+#pragma unroll 1
+        for (int e0 = threadIdx.x; e0 < L.E; e0 += 4 * kTT) {
+            int o[4], q[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int e = min(e0 + k * kTT, L.E - 1);
+                o[k] = __ldcg(L.hoff + e);
+                q[k] = __ldcg(L.hoff + e + 1);
             }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int v = v0 + k * kTT;
-                if (v < N && (v < nlo || v >= nhi)) out[v] = x[k];
+            for (int k = 0; k < 4; ++k) {
+                const int e = e0 + k * kTT;
+                if (e >= L.E) continue;
+                so[e] = (uint16_t)o[k];
+                if (q[k] - o[k] > kThreadPins) tiny_ints(t.wide)[atomicAdd(&s.nwide, 1u)] = e;
+            }
+        }
+        if (threadIdx.x == 0) so[L.E] = (uint16_t)L.P;
+    }
+    __syncthreads();
+}
+
+// One wide hyperedge by a warp (see tiny_edges).
+template <class Pins>
+__device__ __forceinline__ void tiny_wide(Pins pin, const int *hw, const uint8_t *side, int *out, bool gains, int e,
+                                          int b, int d) {
+    const int lane = threadIdx.x & 31;
+    int n1 = 0;
+    if (gains) {
+#pragma unroll 2
+        for (int i = lane; i < d; i += 32) n1 += side[pin(b + i)];
+        n1 = __reduce_add_sync(0xffffffffu, n1);
+        if (n1 == 0 || n1 == d) return;
+    }
+    const int w = hw ? __ldcg(hw + e) : 1;
+    const int x1 = n1 == 1 ? 2 * w : w, x0 = gains && d - n1 == 1 ? 2 * w : w;
+#pragma unroll 2
+    for (int i = lane; i < d; i += 32) {
+        const int u = pin(b + i);
+        atomicAdd(out + u, gains && side[u] ? x1 : x0);
+    }
+}
+
+// K hyperedges of up to kThreadPins pins by a thread (d[k] = 0: none).  The first four pins of all of them are
+// handled straight-line, predicated: a loop per hyperedge costs a chain of shared-memory latencies and a
+// divergence each.
+template <int K, class Pins>
+__device__ __forceinline__ void tiny_some(Pins pin, const int *hw, const uint8_t *side, int *out, bool gains,
+                                          const int *e, const int *b, const int *d) {
+    int u[K][4];
+    unsigned on1[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) u[k][i] = i < d[k] ? pin(b[k] + i) : 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        on1[k] = 0;
+        if (gains) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) on1[k] |= (i < d[k] ? (unsigned)side[u[k][i]] : 0u) << i;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        if (gains) {
+#pragma unroll 1
+            for (int i = 4; i < d[k]; ++i) on1[k] |= (unsigned)side[pin(b[k] + i)] << i;
+        }
+        const int n1 = __popc(on1[k]), n0 = d[k] - n1;
+        if (gains && (n1 == 0 || n0 == 0)) continue;  // uncut: only -w_e, already in -D
+        const int w = hw && d[k] > 0 ? __ldcg(hw + e[k]) : 1;
+        // a pin alone on its side gets 2 w, the others w
+        const int x1 = n1 == 1 ? 2 * w : w, x0 = gains && n0 == 1 ? 2 * w : w;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i < d[k]) atomicAdd(out + u[k][i], on1[k] >> i & 1u ? x1 : x0);
+#pragma unroll 1
+        for (int i = 4; i < d[k]; ++i) atomicAdd(out + pin(b[k] + i), on1[k] >> i & 1u ? x1 : x0);
+    }
+}
+
+// A pass over the level's hyperedges.  With `sides` (offset of the sides): Algorithm 4's gains, the cut
+// hyperedges' contributions added to the gains; without (-1): the weighted degrees.  Hyperedges of up to
+// kThreadPins pins take a thread, wider ones a warp.
+__device__ __noinline__ void tiny_edges(int sides) {
+    Tiny &s = tiny();
+    const int lane = threadIdx.x & 31, E = s.lev.E;
+    const bool gains = sides >= 0;
+    const uint8_t *side = reinterpret_cast<const uint8_t *>(tiny_at(gains ? sides : 0));
+    int *out = tiny_ints(gains ? s.lev.gain : s.lev.deg);
+    const int *hoff = s.lev.hoff, *hw = s.lev.hw;
+    if (s.lev.staged) {
+        const StagedPins pin{reinterpret_cast<const uint16_t *>(tiny_at(s.lev.sp))};
+        const uint16_t *so = reinterpret_cast<const uint16_t *>(tiny_at(s.lev.so));
+        constexpr int K = 4;
+#pragma unroll 1
+        for (int e0 = threadIdx.x; e0 < E; e0 += K * kTT) {
+            int e[K], b[K], d[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                e[k] = e0 + k * kTT;
+                b[k] = e[k] < E ? so[e[k]] : 0;
+                d[k] = e[k] < E ? so[e[k] + 1] - b[k] : 0;
+                if (d[k] > kThreadPins) d[k] = 0;
+            }
+            tiny_some<K>(pin, hw, side, out, gains, e, b, d);
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int i = threadIdx.x >> 5; i < (int)s.nwide; i += kTT / 32) {
+            const int e = tiny_ints(s.lev.wide)[i];
+            tiny_wide(pin, hw, side, out, gains, e, so[e], so[e + 1] - so[e]);
+        }
+    } else {
+        const GlobalPins pin{s.lev.pins};
+        constexpr int K = 2;
+#pragma unroll 1
+        for (int e0 = (int)(threadIdx.x & ~31u); e0 < E; e0 += K * kTT) {
+            int e[K], b[K], d[K], f[K];
+            unsigned todo[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                e[k] = e0 + lane + k * kTT;
+                b[k] = e[k] < E ? __ldcg(hoff + e[k]) : 0;
+                d[k] = e[k] < E ? __ldcg(hoff + e[k] + 1) - b[k] : 0;
+            }
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                todo[k] = __ballot_sync(0xffffffffu, d[k] > kThreadPins);
+                f[k] = d[k] > kThreadPins ? 0 : d[k];
+            }
+            tiny_some<K>(pin, hw, side, out, gains, e, b, f);
+            __syncwarp();
+#pragma unroll 1
+            for (int k = 0; k < K; ++k) {
+                unsigned m = k ? todo[1] : todo[0];
+                while (m) {
+                    const int src = __ffs(m) - 1;
+                    m &= m - 1;
+                    tiny_wide(pin, hw, side, out, gains, __shfl_sync(0xffffffffu, k ? e[1] : e[0], src),
+                              __shfl_sync(0xffffffffu, k ? b[1] : b[0], src), __shfl_sync(0xffffffffu, k ? d[1] : d[0], src));
+                }
             }
         }
     }
     __syncthreads();
-    trace(a, lv, 24);
 }
 
-// Weighted degrees of the block's slice of level L's nodes into R.ds.
-__device__ void tail_degrees(const TailArgs &a, const TLev &L, const Chunks &ch, char *smem, const Refine &R,
-                             int lv) {
-    refine_pass(a, L, ch, smem, R, R.ds, false, false, lv,
-                [&](const Win &w, int e, int b0, int d) {
-                    const int wt = L.hw ? __ldg(L.hw + e) : 1;
-                    for (int i = 0; i < d; ++i) atomicAdd(&R.gp[w.P[b0 + i]], wt);
-                },
-                [&](const Win &w, int e, int b0, int d) {
-                    const int wt = L.hw ? __ldg(L.hw + e) : 1;
-                    for (int i = threadIdx.x & 31; i < d; i += 32) atomicAdd(&R.gp[w.P[b0 + i]], wt);
-                });
-    // the partial array is reused by the next pass once every block has read it
-    csync();
+// Algorithm 4 gains of every node for the sides at `sides`.
+__device__ __forceinline__ void tiny_gains(int sides) {
+    const Tiny &s = tiny();
+    int *gain = tiny_ints(s.lev.gain);
+    const int *deg = tiny_ints(s.lev.deg), N = s.lev.N;
+#pragma unroll 2
+    for (int v = threadIdx.x; v < N; v += kTT) gain[v] = -deg[v];
+    __syncthreads();
+    tiny_edges(sides);
 }
 
-// Algorithm 4 gains of every node of level L for `side` (shared, identical in every block) into
-// R.gf in every block.
-__device__ void tail_gains(const TailArgs &a, const TLev &L, const Chunks &ch, char *smem, const Refine &R,
-                           const uint8_t *side, int lv) {
-    refine_pass(a, L, ch, smem, R, R.gf, true, true, lv,
-                [&](const Win &w, int e, int b0, int d) {
-                    int n1 = 0;
-                    for (int i = 0; i < d; ++i) n1 += side[w.P[b0 + i]];
-                    if (n1 == 0 || n1 == d) return;  // uncut: only -w_e, already in -D
-                    const int wt = L.hw ? __ldg(L.hw + e) : 1;
-                    for (int i = 0; i < d; ++i) {
-                        const int u = w.P[b0 + i];
-                        const int ns = side[u] ? n1 : d - n1;  // pins on u's side
-                        atomicAdd(&R.gp[u], ns == 1 ? 2 * wt : wt);
-                    }
-                },
-                [&](const Win &w, int e, int b0, int d) {
-                    const int lane = threadIdx.x & 31;
-                    int n1 = 0;
-                    for (int i = lane; i < d; i += 32) n1 += side[w.P[b0 + i]];
-                    n1 = warp_sum(n1);
-                    if (n1 == 0 || n1 == d) return;
-                    const int wt = L.hw ? __ldg(L.hw + e) : 1;
-                    for (int i = lane; i < d; i += 32) {
-                        const int u = w.P[b0 + i];
-                        const int ns = side[u] ? n1 : d - n1;
-                        atomicAdd(&R.gp[u], ns == 1 ? 2 * wt : wt);
-                    }
-                });
-}
-
-__device__ void tail_side_weights(const TLev &L, const uint8_t *side, RState *st) {
-    __shared__ unsigned long long red[33];
-    unsigned long long w0 = 0, w1 = 0;
-    for (int v = threadIdx.x; v < L.N; v += kTT) {
-        const unsigned long long w = (unsigned long long)__ldg(L.nw + v);
-        if (side[v]) w1 += w;
-        else w0 += w;
+// The exact radix passes for a threshold in a clamped end bucket (rare).
+__device__ __noinline__ void tiny_exact(int kind, const uint8_t *side, uint32_t *status) {
+    RState *st = &tiny().st;
+    const TinyLevel &t = tiny().lev;
+#pragma unroll 1
+    for (int pass = 0; pass < 3; ++pass) {
+        d_sel_hist_exact(CtaTeam(), t.N, kind, tiny_ints(t.gain), side, tiny_ints(t.nw), st, st->hist, false);
+        d_sel_find_exact(st, status, st->hist);
+        __syncthreads();
     }
-    w0 = block_sum(w0, red);
-    w1 = block_sum(w1, red);
+}
+
+// One selection and its application (Algorithms 3 and 5: the chosen nodes flip and the side weights follow;
+// rebalance: they become keys).  Ties are ranked by id from bitmaps whose words the warps write whole.
+__device__ __noinline__ void tiny_select(int kind, long long sq, int sides, uint32_t *status) {
+    Tiny &s = tiny();
+    const TinyLevel &t = s.lev;
+    RState *st = &s.st;
+    uint8_t *side = reinterpret_cast<uint8_t *>(tiny_at(sides));
+    const int *gain = tiny_ints(t.gain), *nw = tiny_ints(t.nw);
+    const int lane = threadIdx.x & 31, N = t.N;
+    // candidates: gain at least `floor`, on side `want` (-1: either), weight at most `room`
+    const int floor = kind == SEL_REFINE ? 0 : INT_MIN;
+    const int want = kind == SEL_REFINE ? -1 : (kind == SEL_INITIAL ? 1 : st->heavy);
+    const int room = kind == SEL_REBAL ? (int)min(st->room, (long long)INT_MAX) : INT_MAX;
+#pragma unroll 1
+    for (int i = threadIdx.x; i < kHistBins / 2; i += kTT)
+        reinterpret_cast<uint4 *>(&st->hist[0][0])[i] = make_uint4(0, 0, 0, 0);
     if (threadIdx.x == 0) {
-        st->W[0] = w0;
-        st->W[1] = w1;
+        s.ncand = 0;
+        s.wdelta = 0;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int v = threadIdx.x; v < N; v += kTT) {
+        const int g = gain[v], sd = side[v];
+        if (g < floor || (want >= 0 && sd != want) || nw[v] > room) continue;
+        int b = g - kClampLo;
+        b = b < 0 ? 0 : (b > kHistBins - 1 ? kHistBins - 1 : b);
+        atomicAdd(&st->hist[sd][b], 1u);
+    }
+    __syncthreads();
+    find_threshold<kTT>(st, s.find, kind, sq, false, 0, 0);
+    const bool slow = s.find.slow != 0;
+    if (slow) tiny_exact(kind, side, status);
+    const unsigned mode0 = st->g[0].mode, mode1 = st->g[1].mode, thr0 = st->g[0].thr, thr1 = st->g[1].thr;
+    // some: a group whose threshold's ties are not all taken
+    const bool some0 = mode0 == 2 && (slow || st->hist[0][(int)(thr0 ^ 0x80000000u) - kClampLo] > st->g[0].take_eq);
+    const bool some1 = mode1 == 2 && (slow || st->hist[1][(int)(thr1 ^ 0x80000000u) - kClampLo] > st->g[1].take_eq);
+    int moved = 0;
+    const int words = (N + 31) >> 5;
+    // first the nodes above the threshold (and the ties that are all taken), then the ties of lowest ids
+#pragma unroll 1
+    for (int phase = 0; phase < 3; ++phase) {
+        const int i = phase - 1;  // the group whose ties are taken
+        if (phase > 0) {
+            if (!(i ? some1 : some0)) continue;  // block-uniform
+            __syncthreads();
+            unsigned tot;
+            const unsigned ex = block_scan32<kTT>((int)threadIdx.x < words ? (unsigned)__popc(s.tie[i][threadIdx.x]) : 0u,
+                                                  s.red, &tot);
+            if ((int)threadIdx.x < words) s.pre[threadIdx.x] = ex;
+            __syncthreads();
+        }
+#pragma unroll 1
+        for (int q = threadIdx.x >> 5; q < words; q += kTT / 32) {
+            const int v = 32 * q + lane;
+            int sd = i, g = 0, w = 0;
+            bool take = false;
+            if (phase == 0) {
+                bool in = v < N;
+                if (in) {
+                    g = gain[v];
+                    sd = side[v];
+                    w = nw[v];
+                    in = g >= floor && (want < 0 || sd == want) && w <= room;
+                }
+                const unsigned k = gkey(g), mode = sd > 0 ? mode1 : mode0, thr = sd > 0 ? thr1 : thr0;
+                const bool tie = in && mode == 2 && k == thr && (sd > 0 ? some1 : some0);
+                take = in && !tie && (mode == 1 || (mode == 2 && k >= thr));
+                const unsigned b0 = __ballot_sync(0xffffffffu, tie && sd == 0);
+                const unsigned b1 = __ballot_sync(0xffffffffu, tie && sd == 1);
+                if (lane == 0) {
+                    s.tie[0][q] = b0;
+                    s.tie[1][q] = b1;
+                }
+            } else {
+                const unsigned bits = s.tie[i][q];
+                take = (bits >> lane & 1u) && s.pre[q] + (unsigned)__popc(bits & ((1u << lane) - 1u)) < st->g[i].take_eq;
+                if (take) {
+                    g = (int)((i ? thr1 : thr0) ^ 0x80000000u);
+                    w = nw[v];
+                }
+            }
+            if (!take) continue;
+            if (kind == SEL_REBAL) {
+                s.keys[atomicAdd(&s.ncand, 1u)] = (unsigned long long)~gkey(g) << 32 | (unsigned)v;
+            } else {
+                side[v] = (uint8_t)(sd ^ 1);
+                moved += sd ? -w : w;
+            }
+        }
+    }
+    if (kind != SEL_REBAL) {
+        moved = __reduce_add_sync(0xffffffffu, moved);
+        if (lane == 0 && moved) atomicAdd(&s.wdelta, moved);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            st->W[1] += (unsigned long long)(long long)s.wdelta;
+            st->W[0] -= (unsigned long long)(long long)s.wdelta;
+        }
+    }
+    __syncthreads();
+}
+
+// Ordered move of the rebalance (reading C13).
+__device__ __noinline__ void tiny_move(long long sq, int sides) {
+    Tiny &s = tiny();
+    const TinyLevel &t = s.lev;
+    RState *st = &s.st;
+    uint8_t *side = reinterpret_cast<uint8_t *>(tiny_at(sides));
+    const int *nw = tiny_ints(t.nw);
+    const int n = (int)s.ncand, heavy = st->heavy;
+    if (n == 0) {
+        __syncthreads();
+        if (threadIdx.x == 0) st->warn = 1;
+        __syncthreads();
+        return;
+    }
+    // at most kRebalKeys <= kTT keys: one a thread
+    unsigned w = 0, moved;
+    if ((int)threadIdx.x < n) w = (unsigned)nw[(unsigned)s.keys[threadIdx.x]];
+    else if (threadIdx.x < kRebalKeys) s.keys[threadIdx.x] = ~0ull;
+    const unsigned total = block_sum32<kTT>(w, s.red);
+    const int cut = rebal_prefix<kTT>(s.keys, n, sq, st->room, st->need, nw, total, s.red, s.cut, &moved);
+    if ((int)threadIdx.x < cut) side[(unsigned)s.keys[threadIdx.x]] = (uint8_t)(1 - heavy);
+    if (threadIdx.x == 0) {
+        st->W[1 - heavy] += moved;
+        st->W[heavy] -= moved;
     }
     __syncthreads();
 }
@@ -833,10 +1099,10 @@ __device__ void tail_side_weights(const TLev &L, const uint8_t *side, RState *st
 }  // namespace
 
 __global__ void __launch_bounds__(kTT, 1) k_tail(TailArgs a) {
-    extern __shared__ __align__(16) char smem[];
+    extern __shared__ __align__(16) char tail_smem[];
+    char *smem = tail_smem;
     __shared__ TLev lev[kTailMaxLevels + 1];
     __shared__ int s_ce[kTailMaxChunks + 2], s_cp[kTailMaxChunks + 2];
-    __shared__ int s_cnt[2];
     cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
     // the starting level and its chunk table
@@ -891,56 +1157,48 @@ __global__ void __launch_bounds__(kTT, 1) k_tail(TailArgs a) {
         a.info[0] = nl;
         a.info[1] = overflow ? (int)((need + 1048575) >> 20) : 0;  // MiB needed
     }
-    auto pass_bytes = [&](const TLev &L) { return 4.0 * L.E + 4.0 * L.P + (L.hw ? 4.0 * L.E : 0.0) + 8.0 * L.N; };
-    // refinement view of the shared memory (every coarsening access is behind the last barrier)
-    Refine R;
-    R.gp = reinterpret_cast<int *>(smem + kGP);
-    R.gf = reinterpret_cast<int *>(smem + kGF);
-    R.ds = reinterpret_cast<int *>(smem + kDS);
-    R.wl = reinterpret_cast<int *>(smem + kWL);
-    R.cnt = &s_cnt[0];
-    uint8_t *sides[2] = {reinterpret_cast<uint8_t *>(smem + kSA), reinterpret_cast<uint8_t *>(smem + kSB)};
-    signed char *s_grp = reinterpret_cast<signed char *>(smem + kGR);
-    RState *st = reinterpret_cast<RState *>(smem + kST);
-    unsigned long long *keys = reinterpret_cast<unsigned long long *>(smem + kKY);
-    int *list = reinterpret_cast<int *>(smem + kLS);
-    int cur = 0;
-    __syncthreads();
+    csync();  // no block leaves while another may still read its shared memory
+    if (r != 0) return;
     // Algorithm 5 and the rebalance from the coarsest level (after Algorithm 3 there) up to the
-    // starting level
+    // starting level, by this block alone
+    Tiny &s = tiny();
+    RState *st = &s.st;
+    int cur = 0;
+    if (threadIdx.x == 0) {
+        st->heavy = -1;
+        st->warn = 0;
+        st->room = st->need = 0;
+        st->W[0] = 0;
+        st->W[1] = (unsigned long long)a.W;
+    }
+    __syncthreads();
     for (int l = nl; l >= 0; --l) {
         const TLev &L = lev[l];
-        Chunks ch;
-        load_chunks(L, r, C, ch, s_ce, s_cp);
-        tail_degrees(a, L, ch, smem, R, l);
-        bytes += pass_bytes(L);
-        const long long sq = d_ceil_sqrt(L.N);
+        trace(a, l, 20);
+        tiny_load(L);
+        trace(a, l, 21);
+        tiny_edges(-1);
+        trace(a, l, 22);
+        bytes += 4.0 * L.E + 4.0 * L.P + (L.hw ? 4.0 * L.E : 0.0) + 8.0 * L.N;
+        const long long sq = d_ceil_sqrt(L.N), rounds = (long long)L.N + 1;
+        int sides = (int)offsetof(Tiny, side) + cur * (int)sizeof(s.side[0]);
         if (l == nl) {
             // Algorithm 3 (side 0 grown to its share m0 / m, reading G2)
-            uint8_t *side = sides[cur];
-            for (int v = threadIdx.x; v < L.N; v += kTT) side[v] = 1;
-            if (threadIdx.x == 0) {
-                st->rounds = 0;
-                st->list_count = 0;
-                st->slow = 0;
-            }
-            __syncthreads();
-            tail_side_weights(L, side, st);
-            d_initial_cond(st, (long long)L.N + 1, a.status, true, a.m0, a.m);
+#pragma unroll 1
+            for (int v = threadIdx.x; v < L.N; v += kTT) s.side[cur][v] = 1;
+            if (threadIdx.x == 0) d_initial_cond(st, rounds, a.status, true, a.m0, a.m);
             __syncthreads();
             while (st->flag) {
-                tail_gains(a, L, ch, smem, R, side, l);
-                bytes += pass_bytes(L);
-                d_sel_small(L.N, SEL_INITIAL, sq, R.gf, side, L.nw, st, a.status, nullptr, R.gf,
-                            s_grp, st->hist);
-                __syncthreads();
-                d_initial_cond(st, (long long)L.N + 1, a.status, false, a.m0, a.m);
+                tiny_gains(sides);
+                tiny_select(SEL_INITIAL, sq, sides, a.status);
+                if (threadIdx.x == 0) d_initial_cond(st, rounds, a.status, false, a.m0, a.m);
                 __syncthreads();
             }
         } else {
             // projection of the coarser level's sides
-            const uint8_t *coarse = sides[cur];
-            uint8_t *fine = sides[cur ^ 1];
+            const uint8_t *coarse = s.side[cur];
+            uint8_t *fine = s.side[cur ^ 1];
+#pragma unroll 1
             for (int v0 = threadIdx.x; v0 < L.N; v0 += 4 * kTT) {
                 int cm[4];
 #pragma unroll
@@ -951,43 +1209,37 @@ __global__ void __launch_bounds__(kTT, 1) k_tail(TailArgs a) {
             }
             bytes += 4.0 * L.N;
             cur ^= 1;
+            sides = (int)offsetof(Tiny, side) + cur * (int)sizeof(s.side[0]);
             __syncthreads();
         }
-        uint8_t *side = sides[cur];
+#pragma unroll 1
         for (int it = 0; it < a.iters; ++it) {
-            tail_gains(a, L, ch, smem, R, side, l);
-            bytes += pass_bytes(L);
-            d_sel_small(L.N, SEL_REFINE, 0, R.gf, side, L.nw, st, a.status, nullptr, R.gf, s_grp,
-                        st->hist);
-            __syncthreads();
+            tiny_gains(sides);
+            trace(a, l, 24);
+            tiny_select(SEL_REFINE, 0, sides, a.status);
             trace(a, l, 30);
         }
-        tail_side_weights(L, side, st);
-        d_rebal_cond(st, a.limit0, a.limit1, (long long)L.N + 1, a.status, true);
+        if (threadIdx.x == 0) d_rebal_cond(st, a.limit0, a.limit1, rounds, a.status, true);
         __syncthreads();
         while (st->flag) {
-            tail_gains(a, L, ch, smem, R, side, l);
-            bytes += pass_bytes(L);
-            d_sel_small(L.N, SEL_REBAL, sq, R.gf, side, L.nw, st, a.status, list, R.gf, s_grp,
-                        st->hist);
-            __syncthreads();
-            d_rebal_move(R.gf, side, L.nw, list, st, sq, keys);
+            tiny_gains(sides);
+            trace(a, l, 24);
+            tiny_select(SEL_REBAL, sq, sides, a.status);
+            trace(a, l, 30);
+            tiny_move(sq, sides);
+            if (threadIdx.x == 0) d_rebal_cond(st, a.limit0, a.limit1, rounds, a.status, false);
             __syncthreads();
             trace(a, l, 31);
-            d_rebal_cond(st, a.limit0, a.limit1, (long long)L.N + 1, a.status, false);
-            __syncthreads();
         }
     }
-    if (r == 0) {
-        const uint8_t *side = sides[cur];
-        for (int v = threadIdx.x; v < a.N; v += kTT) a.side_out[v] = side[v];
-        if (threadIdx.x == 0) {
-            *a.status0 = st->warn;
-            a.info[2] = (int)((bytes + a.N) / 1024.0);  // KiB, with the side written
-        }
+    const uint8_t *side = s.side[cur];
+    for (int v = threadIdx.x; v < a.N; v += kTT) a.side_out[v] = side[v];
+    if (threadIdx.x == 0) {
+        *a.status0 = st->warn;
+        a.W_out[0] = st->W[0];
+        a.W_out[1] = st->W[1];
+        a.info[2] = (int)((bytes + a.N) / 1024.0);  // KiB, with the side written
     }
-    // no block leaves while another may still read its shared memory
-    csync();
 }
 
 // ------------------------------------------------------------------ host side
@@ -1041,7 +1293,7 @@ bool tail_eligible(const Level &L, int max_new, int flags) {
     return (tail_chunks(L.P) + C - 1) / C + 1 <= kTailMaxChunks;
 }
 
-void run_tail(bipart_graph *g, std::vector<Level *> &levels, const Params &p, const int64_t limit[2],
+void run_tail(bipart_graph *g, std::vector<Level *> &levels, const Params &p, const int64_t limit[2], int64_t W,
               uint8_t *d_side) {
     cudaStream_t s = g->stream;
     Work &w = g->w;
@@ -1085,6 +1337,8 @@ void run_tail(bipart_graph *g, std::vector<Level *> &levels, const Params &p, co
     a.info = tail_info_slot(g);
     a.side_out = d_side;
     a.status0 = bisect_status_word(g);
+    a.W = W;
+    a.W_out = bisect_weights(g);
     a.status = dev_status(g);
     static const bool tracing = std::getenv("BIPART_TAIL_TRACE") != nullptr;
     a.trace = nullptr;

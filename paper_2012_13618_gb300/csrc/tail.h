@@ -13,12 +13,13 @@ namespace bp {
 constexpr int kTailThreads = 512;         // threads per block of the cluster
 constexpr int kTailNodes = 12288;         // largest level (nodes) the tail can start from
 constexpr int64_t kTailMaxPins = 4'000'000;  // ... and pins (its shared-memory chunk table)
-// Default start: the first level of at most this many pins.  A sweep of the start on the 1M-node
-// netlist (graph replay, one GB300) measured 2.694 ms per bisection from 70K pins, 2.73 ms from
-// 170K, 2.86 ms from 420K and 3.17 ms from 800K, against 2.68-2.72 ms with the grid path alone:
-// above ~70K pins the grid's 152 SMs outrun one cluster; below it the tail removes ~50 launches
-// and, in the eager first call, the host round trips of the small levels.
-constexpr int64_t kTailStartPins = 70'000;
+// Default start: the first level of at most this many pins.  Swept as the start (no tail, 4K, 10K, 25K, 45K,
+// 70K pins): 10K-node uniform replays 916, 894, 873, 830, 880, 881 us; 16-way parts of a 250K-node netlist 13.6,
+// 13.0, 13.0, 12.9, 14.2, 16.4 ms; 1M-node netlist 3.12, 3.08, 3.05, 3.01, 3.02, 3.10 ms; a mix of 12 graphs
+// on the server 56.5, 58.5, 57.4, 56.9, 61.7, 73.8 ms; one-shot 1,000 nodes 1177 us without, 740 us from
+// 10K up.  Above ~25K pins a level no longer fits one block's shared memory beside its nodes, and the
+// refinement's passes go back to L2.
+constexpr int64_t kTailStartPins = 25'000;
 constexpr int kTailMaxLevels = 64;        // coarse levels one tail may build
 constexpr int kTailMaxCluster = 16;
 constexpr int kTailChunk = 2048;          // chunk boundaries of a level every this many pins
@@ -51,6 +52,8 @@ struct TailArgs {
                  // [2] algorithmic KiB the launch moved
     uint8_t *side_out;  // bisection of the starting level
     unsigned *status0;  // whether the starting level's rebalance ran out of candidates
+    long long W;        // total node weight
+    unsigned long long *W_out;  // the starting level's side weights
     uint32_t *status;
     unsigned long long *trace;  // diagnostics (BIPART_TAIL_TRACE, eager calls): phase time stamps
 };

@@ -234,9 +234,13 @@ void read_i32s(bipart_graph *g, int n, const int32_t *const *d, int32_t *v) {
         for (int i = 0; i < n; ++i) v[i] = read_i32(g, d[i]);
         return;
     }
-    // the values and the status word in one round trip
-    for (int i = 0; i < n; ++i)
-        BP_CUDA(cudaMemcpyAsync(g->w.host_small + i, d[i], sizeof(int32_t), cudaMemcpyDeviceToHost, g->stream));
+    // The values and the status word in one round trip, neighbouring words in one copy.  What bounds it: ~2 us
+    // of host and copy-engine time a copy; the tail's 78 words are two copies.
+    for (int i = 0, j; i < n; i = j) {
+        for (j = i + 1; j < n && d[j] == d[j - 1] + 1;) ++j;
+        BP_CUDA(cudaMemcpyAsync(g->w.host_small + i, d[i], sizeof(int32_t) * (size_t)(j - i), cudaMemcpyDeviceToHost,
+                                g->stream));
+    }
     BP_CUDA(cudaMemcpyAsync(g->w.host_small + 1023, dev_status(g), sizeof(uint32_t), cudaMemcpyDeviceToHost,
                             g->stream));
     sync(g);
@@ -545,10 +549,8 @@ void extract_subgraph(bipart_graph *g, const int *d_part, int j, bipart_graph *k
         scan(L.E, SubEdgeIn{cnt}, SubEdgeOut{L.E, L.hw(), t_hoff, t_hw, emap, small + 2, nullptr},
              w.scan, dev_status(g), s);
     }
-    BP_CUDA(cudaMemcpyAsync(w.host_small, small, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
-    BP_CUDA(cudaMemcpyAsync(w.host_small + 4, small + 4, sizeof(int), cudaMemcpyDeviceToHost, s));
-    sync(g);
-    check_status(g);
+    BP_CUDA(cudaMemcpyAsync(w.host_small, small, 5 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    check_status(g);  // waits for both copies
     const int N = L.N > 0 ? (int)w.host_small[4] : 0;
     const int E = L.E > 0 ? (int)w.host_small[2] : 0;
     const int P = L.E > 0 ? (int)w.host_small[3] : 0;
@@ -656,11 +658,25 @@ void bisect_body(bipart_graph *g, Level &L0, const Params &p, int64_t W, uint8_t
     if (g->ex.capturing) flush_checks(g);
 }
 
-int read_bisect_status(bipart_graph *g) {
+// The bisection's result (BIPART_OK or BIPART_WARN_IMBALANCED) and the device status word in one round trip.
+int read_bisect_status(bipart_graph *g, uint32_t *dev) {
     BP_CUDA(cudaMemcpyAsync(g->w.host_small, bisect_status_word(g), sizeof(unsigned),
                             cudaMemcpyDeviceToHost, g->stream));
-    sync(g);
+    *dev = read_status_word(g);
     return g->w.host_small[0] ? BIPART_WARN_IMBALANCED : BIPART_OK;
+}
+
+// Where a bisection's sides go: parts[v] (v through l2g, if any) = lo or hi.
+struct PartsOut {
+    const int *l2g;
+    int32_t lo, hi;
+    int *parts;
+};
+
+void write_parts(bipart_graph *g, const uint8_t *d_side, const PartsOut &o) {
+    ProfScope ps("side_to_part", 5.0 * g->L0.N, g->stream);
+    k_side_to_part<<<grid_for(g->L0.N), kBlock, 0, g->stream>>>(g->L0.N, d_side, o.l2g, o.lo, o.hi, o.parts);
+    BP_LAUNCH();
 }
 
 // Captures the bisection just run eagerly (its sizes recorded) into a CUDA graph with WHILE / IF
@@ -734,7 +750,9 @@ bool same_params(const Params &a, const Params &b) {
 // level sizes.  Second call: captures those launches into a CUDA graph and launches it.  Later
 // calls: launch the graph.  A replay whose device-side size checks fail (or a change of buffers
 // or of profiling) drops the plan and runs eagerly again.
-int bisect_top(bipart_graph *g, const Params &p, uint8_t *d_side, int *nlev) {
+// The parts are written behind either, ahead of the one round trip that reads the results (a replay whose
+// checks failed is followed by an eager run, which writes them again).
+int bisect_top(bipart_graph *g, const Params &p, uint8_t *d_side, int *nlev, const PartsOut &out) {
     Plan &pl = g->plan;
     Exec &ex = g->ex;
     g->last_replayed = false;
@@ -758,7 +776,9 @@ int bisect_top(bipart_graph *g, const Params &p, uint8_t *d_side, int *nlev) {
         g->w.scan.dirty[1] = pl.scan_dirty[1];
         if (timing) cudaEventRecord(t1, g->stream);
         for (int64_t i = 0; i < pl.launches; ++i) note_launch();
-        sync(g);
+        write_parts(g, d_side, out);
+        uint32_t st = 0;
+        const int res = read_bisect_status(g, &st);
         if (timing) {
             float ms = 0;
             cudaEventElapsedTime(&ms, t0, t1);
@@ -766,13 +786,12 @@ int bisect_top(bipart_graph *g, const Params &p, uint8_t *d_side, int *nlev) {
             cudaEventDestroy(t0);
             cudaEventDestroy(t1);
         }
-        const uint32_t st = read_status_word(g);
         if (!(st & DEV_PLAN_MISMATCH)) {
-            check_status(g);
+            raise_status(st);
             prof_collect(pl.probes);
             *nlev = pl.nlev;
             g->last_replayed = true;
-            return read_bisect_status(g);
+            return res;
         }
         // the replayed control flow did not match this run: discard the plan, run eagerly
         BP_CUDA(cudaMemsetAsync(dev_status(g), 0, sizeof(uint32_t), g->stream));
@@ -791,8 +810,10 @@ int bisect_top(bipart_graph *g, const Params &p, uint8_t *d_side, int *nlev) {
     }
     ex.recording = false;
     const int64_t kernels = bipart_kernel_launches() - k0;
-    int st = read_bisect_status(g);
-    check_status(g);
+    write_parts(g, d_side, out);
+    uint32_t dev = 0;
+    const int st = read_bisect_status(g, &dev);
+    raise_status(dev);
     ex.rec_valid = true;
     ex.rec_params = p;
     ex.rec_gen = g->gen;
@@ -831,11 +852,10 @@ int refine_kept(bipart_graph *g, int64_t e6, int32_t iters, int *d_parts) {
     }
     if ((int)levels.size() != g->hier.nlev) throw Fail{BIPART_ERR_CUDA, "kept hierarchy changed size"};
     uncoarsen(g, levels, limit, W, p.m0, p.m, p.iters, d_side, tail_from);
-    int st = read_bisect_status(g);
-    k_side_to_part<<<grid_for(L0.N), kBlock, 0, s>>>(L0.N, d_side, nullptr, 0, p.m0, d_parts);
-    BP_LAUNCH();
-    sync(g);
-    check_status(g);
+    write_parts(g, d_side, PartsOut{nullptr, 0, p.m0, d_parts});
+    uint32_t dev = 0;
+    const int st = read_bisect_status(g, &dev);
+    raise_status(dev);
     return st;
 }
 
@@ -859,19 +879,13 @@ int partition_device(bipart_graph *g, const Params &p, int *d_parts) {
     Params top = p;
     top.m = p.k;
     top.m0 = (p.k + 1) / 2;
-    int st = bisect_top(g, top, d_side, &nlev);
+    int st = bisect_top(g, top, d_side, &nlev, PartsOut{nullptr, 0, top.m0, d_parts});
     if (st != BIPART_OK) status = st;
-    {
-        ProfScope ps("side_to_part", 5.0 * L.N, s);
-        k_side_to_part<<<grid_for(L.N), kBlock, 0, s>>>(L.N, d_side, nullptr, 0, top.m0, d_parts);
-        BP_LAUNCH();
-    }
     if (p.k == 2) {
         g->hier.nlev = nlev;
         g->hier.valid = true;
         g->hier.tail_from = g->last_tail_from;
         g->hier.params = top;
-        sync(g);
         return status;
     }
     const int lanes = g->kid_lanes > 0 ? g->kid_lanes : default_lanes();
@@ -945,10 +959,7 @@ int partition_device(bipart_graph *g, const Params &p, int *d_parts) {
                 if (kid->L0.N > 0) {
                     uint8_t *ds = (uint8_t *)kid->side_out.ensure((size_t)kid->L0.N, kid->stream);
                     int nl = 0;
-                    st[(size_t)i] = bisect_top(kid, q, ds, &nl);
-                    k_side_to_part<<<grid_for(kid->L0.N), kBlock, 0, kid->stream>>>(
-                        kid->L0.N, ds, kid->l2g.as<int>(), lo, lo + q.m0, d_parts);
-                    BP_LAUNCH();
+                    st[(size_t)i] = bisect_top(kid, q, ds, &nl, PartsOut{kid->l2g.as<int>(), lo, lo + q.m0, d_parts});
                 }
                 BP_CUDA(cudaEventRecord(kid->kid_done, kid->stream));
             } catch (const Fail &e) {
@@ -978,7 +989,7 @@ int partition_device(bipart_graph *g, const Params &p, int *d_parts) {
             BP_CUDA(cudaMemcpyAsync(pa, d_parts, sizeof(int) * (size_t)L.N, cudaMemcpyDeviceToDevice, s));
         ranges.swap(next);
     }
-    sync(g);
+    check_status(g);
     return status;
 }
 
@@ -1255,7 +1266,6 @@ void finish_create(bipart_graph *g, int32_t N, int32_t E, int32_t P, int64_t W, 
                    const int *d_pins, const int *d_nw, const int *d_hw) {
     build_level0(g, g->L0, N, E, P, d_hoff, d_pins, d_nw, d_hw);
     g->total_node_weight = W;
-    sync(g);
     check_status(g);
 }
 
@@ -1368,7 +1378,6 @@ int graph_partition_host(bipart_graph *g, const Params &p, int32_t *out) {
     int st = partition_device(g, p, d);
     if (N > 0) BP_CUDA(cudaMemcpyAsync(out, d, sizeof(int) * (size_t)N, cudaMemcpyDeviceToHost, g->stream));
     sync(g);
-    check_status(g);
     return st;
 }
 
@@ -1505,7 +1514,7 @@ namespace {
 int partition_to_device(bipart_handle h, const Params &p, int32_t *d_out_parts) {
     if (!d_out_parts && h->L0.N > 0) throw Fail{BIPART_ERR_INVALID_ARG, "out_parts is NULL"};
     int st = partition_device(h, p, d_out_parts);
-    check_status(h);
+    sync(h);
     return st;
 }
 
@@ -1516,7 +1525,6 @@ int partition_to_host(bipart_handle h, const Params &p, int32_t *out_parts) {
     int st = partition_device(h, p, d);
     if (N > 0) BP_CUDA(cudaMemcpyAsync(out_parts, d, sizeof(int) * (size_t)N, cudaMemcpyDeviceToHost, h->stream));
     sync(h);
-    check_status(h);
     return st;
 }
 

@@ -487,12 +487,13 @@ void contract(bipart_graph *g, int32_t E, int32_t P, const int *hoff, const int 
             ProfScope ps("contract_offsets", 16.0 * E, s);
             scan(E, CompactIn{cnt, rep}, out, w.scan, dev_status(g), s);
         }
-        const int32_t *ptr[3] = {sizes, sizes + 1, n_slot};
+        const int32_t *ptr[3] = {n_slot, sizes, sizes + 1};  // n_slot lies before sizes: one copy
         int32_t v[3];
-        read_i32s(g, n_slot ? 3 : 2, ptr, v);
-        c.E = v[0];
-        c.P = v[1];
-        if (n_slot) c.N = v[2];
+        const int first = n_slot ? 0 : 1;
+        read_i32s(g, 3 - first, ptr + first, v + first);
+        if (n_slot) c.N = v[0];
+        c.E = v[1];
+        c.P = v[2];
         {
             // scratch, coarse pins, degree atomics, per-hyperedge offsets
             ProfScope ps("contract_copy", 12.0 * P + 12.0 * E, s);

@@ -28,9 +28,10 @@
 
 namespace bp {
 
-constexpr int kWalkThread = 32;  // long lists: hyperedges up to this degree are walked by one thread,
-constexpr int kWalkWarp = 512;   // up to this one by the warp that met them, wider ones queued
-constexpr int kWalkShort = 8;    // short lists: wider ones are all queued, so that no warp walks several
+constexpr int kMoveBatch = 2;    // incidences of an entry a lane takes: an entry's run is 2 * lanes at most
+static_assert(kMoveRun == 32 * kMoveBatch && kMoveRunShort == 8 * kMoveBatch, "one batch an entry");
+constexpr int kWalkWarp = 512;   // hyperedges up to this degree are walked by the warp that met them, wider ones
+constexpr int kWalkShort = 64;   // queued; in short lists up to this one, so that no warp walks many pins
 
 __device__ __forceinline__ int contrib(int own, int other) { return (own == 1) - (other == 0); }
 
@@ -39,9 +40,9 @@ __device__ __forceinline__ unsigned long long pair_step(int s) {
     return s ? 1ull - (1ull << 32) : (1ull << 32) - 1ull;
 }
 
-// Entry q of a moved node's incidence list (first b, length d), the node now on side s.
-__device__ __forceinline__ int4 move_entry(int v, int b, int d, int q, int s) {
-    return make_int4(v, b + q * kMoveRun, min(b + d, b + (q + 1) * kMoveRun), s);
+// Entry q of a moved node's incidence list (first b, length d), `run` a piece, the node now on side s.
+__device__ __forceinline__ int4 move_entry(int v, int b, int d, int q, int s, int run) {
+    return make_int4(v, b + q * run, b + q * run + min(d - q * run, run), s);
 }
 
 // Adds x0 / x1 to the gains of pins [a, b) on side 0 / 1 of `wside`; thread `t` of `nt`.
@@ -62,6 +63,65 @@ static __device__ __noinline__ void walk_pins(const int *pins, const uint8_t *ws
     }
 }
 
+// A wide hyperedge (pins [a, a + d)) whose changes are x0 / x1, queued for pass 2, one place per kItemPins pins.
+static __device__ __noinline__ void queue_wide(const MoveArgs &m, unsigned *queued, const uint8_t *wside, int a, int d,
+                                               int x0, int x1) {
+    const unsigned items = d > 0 ? (unsigned)(d + kItemPins - 1) / kItemPins : 0u;
+    const unsigned upto = warp_inclusive_scan(items);
+    unsigned base = 0;
+    if ((threadIdx.x & 31) == 31) base = atomicAdd(queued, upto);
+    base = __shfl_sync(0xffffffffu, base, 31) + upto - items;
+#pragma unroll 1
+    for (unsigned i = 0; i < items; ++i) {
+        const int p0 = a + (int)i * kItemPins, p1 = min(p0 + kItemPins, a + d);
+        if (base + i < (unsigned)m.item_cap) m.items[base + i] = make_int4(p0, p1, x0, x1);
+        else walk_pins(m.pins, wside, m.gain, p0, p1, x0, x1, 0, 1);  // a full queue
+    }
+    __syncwarp();
+}
+
+// Every lane's two hyperedges (pins [a, a + d), d = 0: none) add their changes x0 / x1 to their pins.  The warp
+// walks the pins of all lanes as one sequence, 128 in flight: a lane walking its own hyperedge held the
+// others up for the longest one's chain of loads (5M x 5M row-net, level of 461K nodes: pass 1 of a
+// rebalance round 25 us with the wait for the slowest warp, now 11).
+static __device__ __noinline__ void walk_changed(const MoveArgs &m, const uint8_t *wside, int a, int d, int x0, int x1,
+                                                 int b, int f, int z0, int z1) {
+    const int lane = threadIdx.x & 31;
+    const int upto = (int)warp_inclusive_scan((unsigned)(d + f)), first = upto - d - f;
+    const int total = __shfl_sync(0xffffffffu, upto, 31);
+#pragma unroll 1
+    for (int i0 = 0; i0 < total; i0 += 128) {
+        int u[4], s[4], y0[4], y1[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            u[k] = -1;
+            y0[k] = y1[k] = 0;
+            if (i0 + 32 * k >= total) continue;  // warp-uniform
+            const int i = i0 + 32 * k + lane;
+            int l = 0;  // the lane pin i belongs to: the last one whose pins start at or before it
+#pragma unroll
+            for (int h = 16; h > 0; h >>= 1) {
+                const int at = __shfl_sync(0xffffffffu, first, l + h);
+                if (at <= i) l += h;
+            }
+            const int o = i - __shfl_sync(0xffffffffu, first, l), da = __shfl_sync(0xffffffffu, d, l);
+            const int pa = __shfl_sync(0xffffffffu, a, l), pb = __shfl_sync(0xffffffffu, b, l);
+            const int xa0 = __shfl_sync(0xffffffffu, x0, l), xa1 = __shfl_sync(0xffffffffu, x1, l);
+            const int xb0 = __shfl_sync(0xffffffffu, z0, l), xb1 = __shfl_sync(0xffffffffu, z1, l);
+            y0[k] = o < da ? xa0 : xb0;
+            y1[k] = o < da ? xa1 : xb1;
+            if (i < total) u[k] = __ldg(m.pins + (o < da ? pa + o : pb + (o - da)));
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s[k] = u[k] >= 0 ? (int)__ldcg(wside + u[k]) : 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int x = s[k] ? y1[k] : y0[k];
+            if (u[k] >= 0 && x) atomicAdd(m.gain + u[k], x);
+        }
+    }
+}
+
 // Pass 1 over the move list's n entries by warps [warp, warps).  queued: the count of work items (zero
 // before the pass).  wside: the sides the walked pins are read by (prev, or the current sides when moved
 // nodes' gains are not needed any more).  With `full` only the pairs are brought up to date.
@@ -69,65 +129,72 @@ static __device__ __noinline__ void move_pass1(const MoveArgs &m, unsigned n, un
                                   const uint8_t *wside, bool full) {
     const int lane = threadIdx.x & 31;
     const int per = 32 / m.lanes, sub = lane % m.lanes, slot = lane / m.lanes;
-    // a short list is bound by its chain of loads: the offsets are then read beside the atomic
-    const bool early = n <= (unsigned)(2 * warps * per);
-    for (unsigned k0 = (unsigned)warp * per; k0 < n; k0 += (unsigned)warps * per) {
-        const unsigned k = k0 + slot;
-        int j = 0, jb = 0;
-        unsigned long long step = 0;
-        if (k < n) {
-            const int4 en = __ldcg(m.ent + k);
-            j = en.y + sub;
-            jb = en.z;
-            step = pair_step(en.w);
+    // The pass is bound by chains of entry, incidence, atomic, pin and side: a warp has two entries (two incidences
+    // a lane each) in flight and the next two loaded ahead.  Offsets are read beside the atomic unless the list
+    // is long (then by few lanes of many).
+    const bool early = n <= (unsigned)(2 * warps * per), beside = n <= (unsigned)(32 * warps * per);
+    const unsigned stride = (unsigned)warps * per, first = (unsigned)warp * per + slot;
+    int4 next[2];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        next[p] = make_int4(0, 0, 0, 0);
+        if (first + p * stride < n) next[p] = __ldcg(m.ent + first + p * stride);
+    }
+#pragma unroll 1
+    for (unsigned k0 = (unsigned)warp * per; k0 < n; k0 += 2 * stride) {
+        int e[2 * kMoveBatch], a[2 * kMoveBatch], d[2 * kMoveBatch], x0[2 * kMoveBatch], x1[2 * kMoveBatch];
+        unsigned long long step[2], o[2 * kMoveBatch];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const int4 en = next[p];
+            step[p] = pair_step(en.w);
+#pragma unroll
+            for (int u = 0; u < kMoveBatch; ++u) {
+                const int j = en.y + sub + u * m.lanes;
+                e[p * kMoveBatch + u] = j < en.z ? __ldg(m.nadj + j) : -1;
+            }
+            const unsigned k = k0 + slot + (2 + p) * stride;
+            next[p] = make_int4(0, 0, 0, 0);
+            if (k < n) next[p] = __ldcg(m.ent + k);
         }
         if (full) {
-#pragma unroll 4
-            for (; j < jb; j += m.lanes) atomicAdd(m.pair + __ldg(m.nadj + j), step);
+#pragma unroll
+            for (int u = 0; u < 2 * kMoveBatch; ++u)
+                if (e[u] >= 0) atomicAdd(m.pair + e[u], step[u / kMoveBatch]);
             continue;
         }
-        while (__any_sync(0xffffffffu, j < jb)) {
-            int a = 0, d = 0, x0 = 0, x1 = 0;
-            if (j < jb) {
-                const int e = __ldg(m.nadj + j);
-                if (early) a = __ldg(m.hoff + e);
-                const unsigned long long o = atomicAdd(m.pair + e, step), q = o + step;
-                const int o0 = (int)(o >> 32), o1 = (int)(unsigned)o, q0 = (int)(q >> 32), q1 = (int)(unsigned)q;
-                x0 = contrib(q0, q1) - contrib(o0, o1);
-                x1 = contrib(q1, q0) - contrib(o1, o0);
-                if (x0 | x1) {
-                    if (!early) a = __ldg(m.hoff + e);
-                    d = o0 + o1;
-                    const int w = m.hw ? __ldg(m.hw + e) : 1;
-                    x0 *= w;
-                    x1 *= w;
-                }
-            }
-            if (d > 0 && d <= (early ? kWalkShort : kWalkThread)) walk_pins(m.pins, wside, m.gain, a, a + d, x0, x1, 0, 1);
-            // wide hyperedges queued for pass 2, one place per kItemPins pins
-            const unsigned items = d > (early ? kWalkShort : kWalkWarp) ? (unsigned)(d + kItemPins - 1) / kItemPins : 0u;
-            if (__any_sync(0xffffffffu, items != 0)) {
-                const unsigned upto = warp_inclusive_scan(items);
-                unsigned base = 0;
-                if (lane == 31) base = atomicAdd(queued, upto);
-                base = __shfl_sync(0xffffffffu, base, 31) + upto - items;
-#pragma unroll 1
-                for (unsigned i = 0; i < items; ++i) {
-                    const int p0 = a + (int)i * kItemPins, p1 = min(p0 + kItemPins, a + d);
-                    if (base + i < (unsigned)m.item_cap) m.items[base + i] = make_int4(p0, p1, x0, x1);
-                    else walk_pins(m.pins, wside, m.gain, p0, p1, x0, x1, 0, 1);  // a full queue
-                }
-            }
-            unsigned wide = early ? 0u : __ballot_sync(0xffffffffu, d > kWalkThread && d <= kWalkWarp);
-            while (wide) {
-                const int src = __ffs(wide) - 1;
-                wide &= wide - 1;
-                const int wa = __shfl_sync(0xffffffffu, a, src), wd = __shfl_sync(0xffffffffu, d, src);
-                const int y0 = __shfl_sync(0xffffffffu, x0, src), y1 = __shfl_sync(0xffffffffu, x1, src);
-                walk_pins(m.pins, wside, m.gain, wa, wa + wd, y0, y1, lane, 32);
-            }
-            j += m.lanes;
+#pragma unroll
+        for (int u = 0; u < 2 * kMoveBatch; ++u) {
+            a[u] = beside && e[u] >= 0 ? __ldg(m.hoff + e[u]) : 0;
+            o[u] = e[u] >= 0 ? atomicAdd(m.pair + e[u], step[u / kMoveBatch]) : 0ull;
         }
+#pragma unroll
+        for (int u = 0; u < 2 * kMoveBatch; ++u) {
+            d[u] = x0[u] = x1[u] = 0;
+            if (e[u] < 0) continue;
+            const unsigned long long q = o[u] + step[u / kMoveBatch];
+            const int o0 = (int)(o[u] >> 32), o1 = (int)(unsigned)o[u], q0 = (int)(q >> 32), q1 = (int)(unsigned)q;
+            x0[u] = contrib(q0, q1) - contrib(o0, o1);
+            x1[u] = contrib(q1, q0) - contrib(o1, o0);
+            if (x0[u] | x1[u]) {
+                if (!beside) a[u] = __ldg(m.hoff + e[u]);
+                d[u] = o0 + o1;
+                const int w = m.hw ? __ldg(m.hw + e[u]) : 1;
+                x0[u] *= w;
+                x1[u] *= w;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2 * kMoveBatch; ++u) {
+            const bool wide = d[u] > (early ? kWalkShort : kWalkWarp);
+            if (!__any_sync(0xffffffffu, wide)) continue;
+            queue_wide(m, queued, wside, a[u], wide ? d[u] : 0, x0[u], x1[u]);
+            if (wide) d[u] = 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 2 * kMoveBatch; u += 2)
+            if (__any_sync(0xffffffffu, (d[u] | d[u + 1]) != 0))
+                walk_changed(m, wside, a[u], d[u], x0[u], x1[u], a[u + 1], d[u + 1], x0[u + 1], x1[u + 1]);
     }
 }
 

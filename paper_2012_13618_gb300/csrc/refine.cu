@@ -88,10 +88,11 @@ k_node_gain(int N, int P, const int *__restrict__ noff, const int *__restrict__ 
     d_node_gain(GridTeam(), N, P, noff, nadj, pair, hw, side, gain, ts, warp_sum);
 }
 
-// The grid's part of a large move (move_dev.cuh): pass 1, then pass 2.  Above P / kMoveFull moved
-// incidences only the pairs are updated and every gain is recomputed from them.
+// The grid's part of a large move (move_dev.cuh): pass 1, then pass 2.  Above P / kMoveFull (kMoveFullHubs)
+// moved incidences only the pairs are updated and every gain is recomputed from them.
 __device__ __forceinline__ bool move_full(const MoveArgs &m, const LoopRound *rd) {
-    return (long long)__ldcg(&rd->inc) * kMoveFull > (long long)m.P;
+    const int part = (long long)m.P >= (long long)kHubDegree * m.N ? kMoveFullHubs : kMoveFull;
+    return (long long)__ldcg(&rd->inc) * part > (long long)m.P;
 }
 
 __global__ void __launch_bounds__(kBlock) k_move_pairs(MoveArgs m) {
@@ -159,7 +160,10 @@ void refine_level(bipart_graph *g, Level &L, const int *cmap, const uint8_t *coa
     m.items = w.items.as<int4>();
     m.item_cap = kItemCap;
     // nodes with short incidence lists share a warp four at a time
-    m.lanes = (int64_t)L.P <= 16 * (int64_t)L.N ? 8 : 32;
+    const bool short_lists = (int64_t)L.P <= kMoveRunShort * (int64_t)L.N;
+    m.lanes = short_lists ? 8 : 32;
+    m.run = short_lists ? kMoveRunShort : kMoveRun;
+    m.run_shift = short_lists ? 4 : 6;
     p.sq = ceil_sqrt64(L.N);
     if (p.sq > kRebalMax) throw Fail{BIPART_ERR_OOM, "level too large for the ordered rebalance"};
     auto *cand = (unsigned long long *)w.list.ensure(sizeof(unsigned long long) * (size_t)std::max<int64_t>(p.sq, 1), s);
@@ -226,7 +230,9 @@ void uncoarsen(bipart_graph *g, std::vector<Level *> &levels, const int64_t limi
     side_buffer(w.side_prev, nmax, s);
     w.gain.ensure(sizeof(int) * (size_t)nmax + 16, s);
     w.pair.ensure(sizeof(unsigned long long) * (size_t)emax, s);
-    w.ent.ensure(sizeof(int4) * (size_t)(nmax + pmax / kMoveRun + 1), s);
+    static_assert(kMoveRunShort == 16 && kMoveRun == 64, "run_shift");
+    // a level with short runs has at most kMoveRunShort incidences a node
+    w.ent.ensure(sizeof(int4) * (size_t)(nmax + std::max<int64_t>(pmax / kMoveRun, nmax) + 1), s);
     w.items.ensure(sizeof(int4) * (size_t)kItemCap, s);
 
     LoopParams p{};

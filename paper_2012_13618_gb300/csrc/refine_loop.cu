@@ -62,6 +62,7 @@ constexpr int kWin = 32 * kWinWords;
 constexpr int kListCap = 4096;           // candidates a block keeps from its pass over the nodes
 constexpr int kStep = 8 * kT;            // nodes a block visits between two flushes of the chosen
 constexpr int kChosenCap = kStep + 4096;
+constexpr int kScan = 4 * kStep;         // nodes a block looks through at once for the few above a guess
 constexpr int kHubs = 64;                // chosen nodes whose long entry lists the block writes together
 
 // The block's view of a launch.  Solo: this block selects for the whole level (the other blocks of the
@@ -209,7 +210,7 @@ __device__ __forceinline__ unsigned warp_places(unsigned *count, unsigned n) {
 }
 
 // The chosen nodes join the level's lists: the rebalance's candidates, or (flipped already) the move
-// list, one entry per kMoveRun incidences and at least one per node.  All threads.
+// list, one entry per m.run incidences and at least one per node.  All threads.
 __device__ __noinline__ void flush_chosen(int kind) {
     Shared &s = sh();
     const MoveArgs &m = s.a.m;
@@ -238,7 +239,7 @@ __device__ __noinline__ void flush_chosen(int kind) {
                 inc += (unsigned)d;
                 const int w = __ldg(m.nw + v);
                 weight += sd ? w : -w;
-                c = d > 0 ? (d + kMoveRun - 1) / kMoveRun : 1;
+                c = d > 0 ? (int)(((unsigned)d + (unsigned)m.run - 1u) >> m.run_shift) : 1;
             }
             unsigned tot;
             const unsigned ex = block_scan32<kT>((unsigned)c, s.red, &tot);
@@ -264,14 +265,15 @@ __device__ __noinline__ void flush_chosen(int kind) {
             }
             if (mine)
 #pragma unroll 1
-                for (int q = 0; q < c; ++q) m.ent[o + q] = move_entry(v, b, d, q, sd);
+                for (int q = 0; q < c; ++q) m.ent[o + q] = move_entry(v, b, d, q, sd, m.run);
             __syncthreads();
             const int hubs = (int)min(s.nhub, (unsigned)kHubs);
 #pragma unroll 1
             for (int h = 0; h < hubs; ++h) {
                 const int hv = s.hub[h].x, hb = __ldg(m.noff + hv), hd = __ldg(m.noff + hv + 1) - hb;
 #pragma unroll 1
-                for (int q = threadIdx.x; q * kMoveRun < hd; q += kT) m.ent[s.hub_at[h] + q] = move_entry(hv, hb, hd, q, s.hub[h].y);
+                for (int q = threadIdx.x; q < (int)(((unsigned)hd + (unsigned)m.run - 1u) >> m.run_shift); q += kT)
+                    m.ent[s.hub_at[h] + q] = move_entry(hv, hb, hd, q, s.hub[h].y, m.run);
             }
             __syncthreads();
         }
@@ -483,6 +485,83 @@ __device__ __noinline__ void exact_threshold(int kind, bool need_w) {
     }
 }
 
+// select_nodes' pass of a rebalance round that starts from a guess, on blocks of more than one step: the ties at
+// the guess go into the bitmap (their number is returned), the nodes above it into the histogram and the
+// list.  Gains and sides of 32 nodes a thread are in flight, then the weights where one of four is on the
+// heavy side and high enough; visit_nodes, with eight and a third load behind the sides, took 2,800 cycles for every
+// 4,096 nodes of a block (round on 461K nodes: 21 thousand cycles of 83, now 11 with the wait for the slowest block).
+__device__ __noinline__ unsigned scan_guess(int gv, int heavy, int room) {
+    Shared &s = sh();
+    constexpr int kQ = kScan / (4 * kT);  // quads of consecutive nodes a thread
+    const int lo = s.x.lo, hi = s.x.hi;
+    const int *gain = s.a.m.gain, *nw = s.a.m.nw;
+    const uint8_t *side = s.a.m.side;
+    const unsigned want = heavy ? 0x01010101u : 0u;
+    const bool wvec = s.x.wvec;
+    unsigned mine = 0;
+#pragma unroll 1
+    for (int v0 = lo; v0 < hi; v0 += kScan) {
+        int4 g[kQ], w[kQ];
+        unsigned in = 0;  // four bits a quad
+#pragma unroll
+        for (int k = 0; k < kQ; ++k) {
+            const unsigned v = (unsigned)v0 + 4u * (threadIdx.x + (unsigned)(k * kT));
+            g[k] = make_int4(INT_MIN, INT_MIN, INT_MIN, INT_MIN);
+            w[k].x = (int)~want;  // the sides, until the weights are here
+            if (v < (unsigned)hi) {
+                g[k] = __ldcg(reinterpret_cast<const int4 *>(gain + v));
+                w[k].x = (int)__ldcg(reinterpret_cast<const unsigned *>(side + v));
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kQ; ++k) {
+            const int v = v0 + 4 * ((int)threadIdx.x + k * kT);
+            const unsigned off = (unsigned)w[k].x ^ want;  // a zero byte: on the side
+            if (g[k].x >= gv && (off & 0xffu) == 0) in |= 1u << (4 * k);
+            if (g[k].y >= gv && (off & 0xff00u) == 0 && v + 1 < hi) in |= 2u << (4 * k);
+            if (g[k].z >= gv && (off & 0xff0000u) == 0 && v + 2 < hi) in |= 4u << (4 * k);
+            if (g[k].w >= gv && (off & 0xff000000u) == 0 && v + 3 < hi) in |= 8u << (4 * k);
+            w[k] = make_int4(0, 0, 0, 0);
+            if (in >> (4 * k) & 15u) {
+                if (wvec) w[k] = __ldg(reinterpret_cast<const int4 *>(nw + v));
+                else w[k] = make_int4(__ldg(nw + v), __ldg(nw + v + 1), __ldg(nw + v + 2), __ldg(nw + v + 3));
+            }
+        }
+        if (!__any_sync(0xffffffffu, in != 0)) continue;
+#pragma unroll
+        for (int k = 0; k < kQ; ++k) {
+            if (!__any_sync(0xffffffffu, (in >> (4 * k) & 15u) != 0)) continue;
+            const int v = v0 + 4 * ((int)threadIdx.x + k * kT);
+            unsigned q = in >> (4 * k) & 15u;
+            if (w[k].x > room) q &= ~1u;
+            if (w[k].y > room) q &= ~2u;
+            if (w[k].z > room) q &= ~4u;
+            if (w[k].w > room) q &= ~8u;
+            const unsigned tie = q & ((g[k].x == gv ? 1u : 0u) | (g[k].y == gv ? 2u : 0u) | (g[k].z == gv ? 4u : 0u) | (g[k].w == gv ? 8u : 0u));
+            if (tie) {
+                mine += (unsigned)__popc(tie);
+                atomicOr(&s.bits[heavy][(v - lo) >> 5], tie << ((v - lo) & 31));
+            }
+            q &= ~tie;
+            if (!__any_sync(0xffffffffu, q != 0)) continue;
+            unsigned o = warp_places(&s.nlist, (unsigned)__popc(q));
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int x = c == 0 ? g[k].x : (c == 1 ? g[k].y : (c == 2 ? g[k].z : g[k].w));
+                if (q >> c & 1u) {
+                    int b = x - kClampLo;
+                    b = b < 0 ? 0 : (b > kHistBins - 1 ? kHistBins - 1 : b);
+                    atomicAdd(&s.st.hist[heavy][b], 1u);
+                    if (o < (unsigned)kListCap) s.list[o] = make_int2((v + c) | (int)((unsigned)heavy << 31), x);
+                    ++o;
+                }
+            }
+        }
+        __syncwarp();
+    }
+    return mine;
+}
+
 // One selection of Algorithm 3 (SEL_INITIAL), Algorithm 5 (SEL_REFINE) or the rebalance (SEL_REBAL)
 // and its application, by the selecting blocks.  The histogram and the lists of x.p ^ 1 are clear.
 //
@@ -505,6 +584,8 @@ __device__ __noinline__ void select_nodes(int kind) {
         const Filter f = filter(kind, st, kind == SEL_REFINE ? 0 : (guess ? gv : INT_MIN));
         clear_pass(one_win ? words : 0);
         unsigned mine = 0;  // ties met
+        if (guess && hi - lo > kStep) mine = scan_guess(gv, heavy, f.room);
+        else
         visit_nodes(lo, hi, f.floor, need_w, a.m.side, [&](const Step &t) {
             unsigned cand = 0, at = 0;
 #pragma unroll

@@ -11,7 +11,9 @@ namespace bp {
 
 constexpr int kLoopThreads = 512;       // threads per block of the cluster
 constexpr int kLoopMaxCluster = 16;
-constexpr int kMoveRun = 64;            // incidences of a moved node one entry of the move list covers
+// Incidences of a moved node one entry of the move list covers: two a lane, for 32 lanes an entry or 8.  With
+// 64 for 8 lanes too a warp went through a node of high degree in four batches while others had none.
+constexpr int kMoveRun = 64, kMoveRunShort = 16;
 constexpr int kItemPins = 128;          // pins of a wide hyperedge one work item covers (four a lane)
 constexpr int kItemCap = 1 << 16;       // work items a pass may queue (beyond: walked on the spot)
 // Moves of more than this many incidences are brought into the gains by the whole grid instead of
@@ -23,8 +25,11 @@ constexpr int kLoopStartPins = 1 << 17;
 // Levels of at most this many nodes are selected by the cluster's first block alone, the others helping
 // with the gain updates only.
 constexpr int kLoopSoloNodes = 4096;
-// Above P / kMoveFull moved incidences every gain is recomputed instead of updated.
-constexpr int kMoveFull = 8;
+// Above P / kMoveFull moved incidences every gain is recomputed instead of updated; above P / kMoveFullHubs
+// where a node has kHubDegree incidences or more on average (the updates' atomics then meet on few
+// nodes).  5M x 5M row-net, us of updates a level at P / 8, P / 32, P / 128: 1370 incidences a node 1779,
+// 2010, 2475; 2460 a node 2398, 1988, 2023; 4100 a node 2779, 2002, 1274; 5800 a node 3275, 1567, 1063.
+constexpr int kMoveFull = 8, kMoveFullHubs = 128, kHubDegree = 2048;
 
 // What one selection leaves for the update after it; two are used in turn.
 struct LoopRound {
@@ -62,7 +67,8 @@ struct MoveArgs {
     int4 *ent;  // move list: node and its side now, incidences [y, z) (move_entry)
     int4 *items;
     int item_cap;
-    int lanes;  // lanes per entry of the move list (8 or 32)
+    int lanes;           // lanes per entry of the move list (8 or 32)
+    int run, run_shift;  // incidences per entry (a power of two) and its logarithm
 };
 
 struct LoopParams {

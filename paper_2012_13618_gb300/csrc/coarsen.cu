@@ -66,8 +66,9 @@ __global__ void __launch_bounds__(kBigThreads, 3)
 k_seg_big(const int *__restrict__ hoff, const int *__restrict__ pins, const int *__restrict__ cmap,
           int *__restrict__ scratch, int *__restrict__ cnt, const int *__restrict__ list,
           const int *__restrict__ counters) {
+    static_assert(kBigThreads == 512, "block_sort's smallest size");
     __shared__ uint32_t bits[kBigWords];
-    d_seg_big<MAP>(GridTeam(), hoff, pins, cmap, scratch, cnt, list, counters, bits);
+    d_seg_big<MAP, GridTeam, true>(GridTeam(), hoff, pins, cmap, scratch, cnt, list, counters, bits);
 }
 
 // Mid and big tiers in one launch (small levels, where the launch is the larger cost; on large
@@ -124,8 +125,14 @@ __device__ __forceinline__ void d_level_init(const LevelInit &li) {
 // Coarse levels with at most kPrivNodes nodes count degrees and claim incidence positions in
 // block-private shared-memory counters: few nodes means many pins per node, and one global
 // atomic per pin would serialise on the heaviest nodes.  Each block merges its counts with one
-// global atomic per node it touched.
-constexpr int kPrivNodes = 24576;
+// global atomic per node it touched.  Up to kPrivNodes nodes two blocks fit an SM; up to kPrivNodesWide one
+// does, which pays where nodes have many pins (5M x 5M row-net, level of 27,393 nodes and 37.5M pins: copy 1992
+// us with global atomics and 210 so, fill 1826 and 494) and not where the merges outnumber the pins (1M-node
+// netlist, 54,019 nodes of 49 pins).
+constexpr int kPrivNodes = 24576, kPrivNodesWide = 52 * 1024, kPrivWideDegree = 256;
+inline bool use_priv(int N, int64_t P) {
+    return N <= kPrivNodes || (N <= kPrivNodesWide && P >= (int64_t)kPrivWideDegree * N);
+}
 constexpr int kPrivBlock = 1024;  // large blocks: clearing and merging N counters is per block
 
 __global__ void __launch_bounds__(kPrivBlock)
@@ -194,10 +201,20 @@ k_fill_adj_priv(int E, int P, int N, const int *__restrict__ hoff, const int *__
 }
 
 // Blocks for the private-counter kernels: one tile of kPrivBlock * kLbItems pins each, at most
-// two blocks per SM (up to 96 KB of counters each); blocks loop over further tiles.
-inline int priv_grid(int P) {
+// two blocks per SM (up to 96 KB of counters each), one for wider levels; blocks loop over further tiles.
+inline int priv_grid(int P, int N) {
     int64_t b = ((int64_t)P + kPrivBlock * kLbItems - 1) / (kPrivBlock * kLbItems);
-    return (int)std::max<int64_t>(1, std::min<int64_t>(b, 2 * 152));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(b, N <= kPrivNodes ? 2 * 152 : 152));
+}
+
+// A CSR's tile starts by search, one thread a tile.  The scan that writes the offsets marks them too, but the
+// thread of a node marks all its tiles, and on levels of few nodes the heaviest one's are most of the launch
+// (5M x 5M row-net, 27,393 nodes: 125 us marked, 16 searched; 461K nodes of 106 incidences: 26).
+constexpr int kSearchTilesDegree = 128;
+__global__ void __launch_bounds__(kBlock) k_search_tiles(int N, int P, const int *__restrict__ noff, int *__restrict__ ts) {
+    const int tiles = (int)(((int64_t)P + kTsGran - 1) / kTsGran);
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < tiles; t += gridDim.x * blockDim.x)
+        ts[t] = lb_seg(noff, t * kTsGran, 0, N - 1);
 }
 
 __global__ void k_fill(int n, int val, int *__restrict__ a) {
@@ -497,8 +514,8 @@ void contract(bipart_graph *g, int32_t E, int32_t P, const int *hoff, const int 
         {
             // scratch, coarse pins, degree atomics, per-hyperedge offsets
             ProfScope ps("contract_copy", 12.0 * P + 12.0 * E, s);
-            if (c.N <= kPrivNodes)
-                k_seg_copy_priv<<<priv_grid(P), kPrivBlock, sizeof(int) * (size_t)std::max(c.N, 1), s>>>(
+            if (use_priv(c.N, c.P))
+                k_seg_copy_priv<<<priv_grid(P, c.N), kPrivBlock, sizeof(int) * (size_t)std::max(c.N, 1), s>>>(
                     E, P, c.N, hoff, scratch, cnt, emap, c.hoff(), c.pins(), deg, ts_in);
             else
                 k_seg_copy<<<lb_grid(P), kLbBlock, 0, s>>>(E, P, hoff, scratch, cnt, emap, c.hoff(), c.pins(), deg,
@@ -541,13 +558,18 @@ void build_incidence_and_init(bipart_graph *g, Level &L, const LevelInit &next) 
     L.b_tsn.ensure(sizeof(int) * ((size_t)L.P / kTsGran + 2), s);
     {
         ProfScope ps("incidence_offsets", 12.0 * L.N, s);
-        scan(L.N, DegIn{deg}, DegOut{L.N, L.noff(), cursor, L.tsn()}, w.scan,
+        const bool search = (int64_t)L.P >= (int64_t)kSearchTilesDegree * L.N;
+        scan(L.N, DegIn{deg}, DegOut{L.N, L.noff(), cursor, search ? nullptr : L.tsn()}, w.scan,
              dev_status(g), s);
+        if (search) {
+            k_search_tiles<<<grid_for(ceil_div_i(L.P, kTsGran)), kBlock, 0, s>>>(L.N, L.P, L.noff(), L.tsn());
+            BP_LAUNCH();
+        }
     }
     if (L.P > 0) {
         ProfScope ps("incidence_fill", 12.0 * L.P + 4.0 * L.E + 32.0 * next.E + 8.0 * next.N, s);
-        if (L.N <= kPrivNodes)
-            k_fill_adj_priv<<<priv_grid(L.P), kPrivBlock, sizeof(int) * (size_t)L.N, s>>>(
+        if (use_priv(L.N, L.P))
+            k_fill_adj_priv<<<priv_grid(L.P, L.N), kPrivBlock, sizeof(int) * (size_t)L.N, s>>>(
                 L.E, L.P, L.N, L.hoff(), L.pins(), cursor, L.nadj(), L.tsh(), next);
         else
             k_fill_adj<<<lb_grid(L.P), kLbBlock, 0, s>>>(L.E, L.P, L.hoff(), L.pins(), cursor, L.nadj(),
@@ -678,7 +700,7 @@ void coarsen_init() {
     static std::once_flag once;
     static cudaError_t err = cudaSuccess;
     std::call_once(once, []() {
-        const int bytes = (int)(sizeof(int) * kPrivNodes);
+        const int bytes = (int)(sizeof(int) * kPrivNodesWide);
         err = cudaFuncSetAttribute(k_seg_copy_priv, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (err == cudaSuccess)
             err = cudaFuncSetAttribute(k_fill_adj_priv, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);

@@ -18,6 +18,7 @@ constexpr int kGridMidDeg = 256;  // the same bound for the grid kernels, where 
                                   // up to 1024 keys would hold up the whole launch
 constexpr int kBigWords = 8192;   // bitmap window of the block tier: 32 KB = 262,144 ids
 constexpr int kBigCache = 12;     // mapped pins a block-tier thread keeps in registers
+constexpr int kBigAhead = 4;      // and of the pins beyond, gathered together
 
 // ------------------------------------------------------------------ small fixed sorting network
 template <int n>
@@ -171,11 +172,53 @@ __device__ void d_seg_mid(Team t, const int *hoff, const int *pins, const int *c
     }
 }
 
+// Ascending bitonic sort of n2 keys (a power of two, at least 64) in shared memory by the block.  Steps whose
+// pairs lie within 64 consecutive keys stay within one warp's pairs.
+static __device__ __noinline__ void block_sort(uint32_t *key, int n2) {
+#pragma unroll 1
+    for (int size = 2; size <= n2; size <<= 1) {
+#pragma unroll 1
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+#pragma unroll 4
+            for (int i = threadIdx.x; i < n2 / 2; i += blockDim.x) {
+                const int at = 2 * i - (i & (stride - 1));
+                const uint32_t a = key[at], b = key[at + stride];
+                if ((a > b) == ((at & size) == 0)) {
+                    key[at] = b;
+                    key[at + stride] = a;
+                }
+            }
+            // the next step's pairs: this step's warps own them unless its stride, or the next size's, is wider
+            if (stride > 32 || (stride == 1 && size >= 64)) __syncthreads();
+            else __syncwarp();
+        }
+    }
+}
+
+// Distinct values of the d keys in `key` (sorted here; padded to a power of two) to out, ascending; returns
+// their number.  All threads.
+static __device__ __noinline__ int block_unique(uint32_t *key, int d, int n2, int *out, int *red) {
+    block_sort(key, n2);
+    __syncthreads();
+    const int per = n2 / (int)blockDim.x > 0 ? n2 / (int)blockDim.x : 1, i0 = (int)threadIdx.x * per;
+    int c = 0;
+    for (int i = i0; i < i0 + per && i < d; ++i) c += i == 0 || key[i] != key[i - 1];
+    int tot;
+    int pos = block_exclusive_scan<int>(c, red, &tot);
+    for (int i = i0; i < i0 + per && i < d; ++i)
+        if (i == 0 || key[i] != key[i - 1]) out[pos++] = (int)key[i];
+    return tot;
+}
+
 // Big tier: one block per listed hyperedge (d > 1024).  Distinct values are found with a
 // shared-memory bitmap `bits` (kBigWords words) over a window of ids [lo, lo + 32 * kBigWords);
 // windows sweep the range [min, max] of the mapped pins, so the output comes out ascending
 // without a sort.
-template <bool MAP, class Team>
+//
+// kSort: hyperedges whose pins spread over several windows and fit the bitmap's memory as keys are sorted
+// instead.  A window costs its clearing, counting and emission whatever it holds (5M x 5M row-net, first level:
+// 7 windows for 11 thousand rows of more than 256 pins: 4.7 ms in this tier and the smaller ones, 2.1 with the sort).
+template <bool MAP, class Team, bool kSort = false>
 __device__ void d_seg_big(Team t, const int *hoff, const int *pins, const int *cmap, int *scratch,
                           int *cnt, const int *list, const int *counters, uint32_t *bits) {
     __shared__ int red[33];
@@ -201,10 +244,18 @@ __device__ void d_seg_big(Team t, const int *hoff, const int *pins, const int *c
                 hi = max(hi, xs[k]);
             }
         }
-        for (int i = cached + threadIdx.x; i < d; i += blockDim.x) {
-            int x = mapped<MAP, Team>(pins, cmap, a + i);
-            lo = min(lo, x);
-            hi = max(hi, x);
+        for (int i0 = cached + threadIdx.x; i0 < d; i0 += kBigAhead * blockDim.x) {
+            int m[kBigAhead];
+#pragma unroll
+            for (int k = 0; k < kBigAhead; ++k) {
+                const int i = i0 + k * (int)blockDim.x;
+                m[k] = mapped<MAP, Team>(pins, cmap, a + (i < d ? i : i0));
+            }
+#pragma unroll
+            for (int k = 0; k < kBigAhead; ++k) {
+                lo = min(lo, m[k]);
+                hi = max(hi, m[k]);
+            }
         }
         lo = warp_min(lo);
         hi = warp_max(hi);
@@ -215,6 +266,25 @@ __device__ void d_seg_big(Team t, const int *hoff, const int *pins, const int *c
         lo = s_minmax[0];
         hi = s_minmax[1];
         int written = 0;
+        if constexpr (kSort) {
+            const int64_t windows = ((int64_t)hi - lo) / (32 * kBigWords) + 1;
+            if (windows > 1 && d <= kBigWords && (windows > 3 || d <= kBigWords / 2)) {  // block-uniform
+                int n2 = 512;
+                while (n2 < d) n2 <<= 1;
+#pragma unroll
+                for (int k = 0; k < kBigCache; ++k) {
+                    const int i = threadIdx.x + k * (int)blockDim.x;
+                    if (i < n2) bits[i] = i < d ? (uint32_t)xs[k] : 0xffffffffu;
+                }
+                for (int i = cached + threadIdx.x; i < n2; i += blockDim.x)
+                    bits[i] = i < d ? (uint32_t)mapped<MAP, Team>(pins, cmap, a + i) : 0xffffffffu;
+                __syncthreads();
+                written = block_unique(bits, d, n2, scratch + a, red);
+                if (threadIdx.x == 0) cnt[e] = written;
+                __syncthreads();
+                continue;
+            }
+        }
         for (int64_t wlo = lo; wlo <= hi; wlo += 32 * kBigWords) {
             const int64_t rest = (int64_t)hi - wlo + 1;
             const int64_t span = rest < 32 * (int64_t)kBigWords ? rest : 32 * (int64_t)kBigWords;
@@ -227,9 +297,18 @@ __device__ void d_seg_big(Team t, const int *hoff, const int *pins, const int *c
                 if (threadIdx.x + k * (int)blockDim.x < d && x >= 0 && x < span)
                     atomicOr(&bits[x >> 5], 1u << (x & 31));
             }
-            for (int i = cached + threadIdx.x; i < d; i += blockDim.x) {
-                int64_t x = (int64_t)mapped<MAP, Team>(pins, cmap, a + i) - wlo;
-                if (x >= 0 && x < span) atomicOr(&bits[x >> 5], 1u << (x & 31));
+            for (int i0 = cached + threadIdx.x; i0 < d; i0 += kBigAhead * blockDim.x) {
+                int m[kBigAhead];
+#pragma unroll
+                for (int k = 0; k < kBigAhead; ++k) {
+                    const int i = i0 + k * (int)blockDim.x;
+                    m[k] = i < d ? mapped<MAP, Team>(pins, cmap, a + i) : -1;
+                }
+#pragma unroll
+                for (int k = 0; k < kBigAhead; ++k) {
+                    const int64_t x = (int64_t)m[k] - wlo;  // -1 lies before every window
+                    if (x >= 0 && x < span) atomicOr(&bits[x >> 5], 1u << (x & 31));
+                }
             }
             __syncthreads();
             // each thread owns a contiguous run of words; block scan of their popcounts

@@ -427,7 +427,7 @@ __device__ void d_fill_adj_with(Team t, int E, int P, const int *hoff, const int
 #pragma unroll
         for (int k = 0; k < kLbItems; ++k) {
             if (k < n) {
-                while (j + k >= send) { ++s; send = end(s); }
+                if (j + k >= send) s = lb_next(s, j + k, end, send);
                 e[k] = s;
                 v[k] = Team::ld(pins + j + k);
             }

@@ -702,8 +702,7 @@ def run_once(replay=False):
             WORKLOAD["refine_iters"])
     st = h.partition_device(*args)
     if replay:
-        # the second call records every level on the grid (when the first used the cluster tail)
-        # and the third captures the plan; the call in the range replays it
+        # the second call captures the plan and replays it, like the third; so does the call in the range
         h.partition_device(*args)
         h.partition_device(*args)
         torch.cuda.synchronize()

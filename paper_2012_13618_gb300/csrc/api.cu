@@ -679,8 +679,8 @@ void write_parts(bipart_graph *g, const uint8_t *d_side, const PartsOut &o) {
     BP_LAUNCH();
 }
 
-// Captures the bisection just run eagerly (its sizes recorded) into a CUDA graph with WHILE / IF
-// nodes for the device-driven loops.  Best effort: on any failure the plan stays invalid and the
+// Captures the bisection just run eagerly (its sizes and decisions recorded) into a straight-line CUDA graph
+// whose checks find a replay that does not match.  Best effort: on any failure the plan stays invalid and the
 // next call runs eagerly again.
 void capture_plan(bipart_graph *g, const Params &p, uint8_t *d_side, int nlev, int64_t kernels) {
     Plan &pl = g->plan;

@@ -6,13 +6,13 @@
 // five to eight kernels of 4-25 us plus, outside a captured plan, two host round trips, and every round
 // recounted all pins.  Here the steps are separated by cluster barriers (0.5-0.7 us with their L2 round
 // trip), the gains are updated from the moved nodes (move_dev.cuh), and every decision is computed by
-// every block from the same data, so nothing is read back.  Replayed bisections, before and after:
-// 5M x 5M row-net 232 -> 72 ms (600 rebalance rounds: 513 -> 50 us each on the level of 461K nodes and 49M
-// pins), 1M-node netlist 3.30 -> 2.99 ms, 90K-node netlist with weighted nets 2.10 -> 1.65 ms.
+// every block from the same data, so nothing is read back.  Bisections of the versions before and now:
+// 5M x 5M row-net 237 -> 53 ms (600 rebalance rounds: 513 -> 33 us each on the level of 461K nodes and 49M
+// pins), 1M-node netlist 3.4 -> 2.8 ms, 90K-node netlist with weighted nets 2.7 -> 1.8 ms.
 //
 // 512 threads a block: the passes of small levels are bound by the latency of their collectives, which
-// 1024 threads made 1.2x slower; the cluster (one GPC) streams node arrays at about 0.8 TB/s, enough for
-// levels of up to a few million nodes (5M nodes: 0.15 ms a selection).
+// 1024 threads made 1.2x slower.  The cluster (one GPC) streams node arrays at a few hundred GB/s; where a
+// refinement selection is bound by that the grid takes it (k_sel_count in refine.cu).
 //
 // Work split: on large levels block r of C owns the node range [r R, (r + 1) R) for the passes over
 // nodes (the ranges ascend, so ties are ranked by id from per-block counts); on small ones the
@@ -47,7 +47,7 @@ struct LoopArgs {
     long long W, limit0, limit1, sq, max_rounds;
     int m0, mt;                // Algorithm 3: side 0 grows to m0 / mt of the weight
     int iters;
-    bool initial, resume, suspend, solo;
+    bool initial, resume, pending, suspend, solo;
     bool start;                // project the sides and count the gains first (small levels)
     const int *cmap;           // start: node -> node of the coarser level (null: all nodes on side 1)
     const uint8_t *coarse;
@@ -63,7 +63,8 @@ constexpr int kListCap = 4096;           // candidates a block keeps from its pa
 constexpr int kStep = 8 * kT;            // nodes a block visits between two flushes of the chosen
 constexpr int kChosenCap = kStep + 4096;
 constexpr int kScan = 4 * kStep;         // nodes a block looks through at once for the few above a guess
-constexpr int kHubs = 64;                // chosen nodes whose long entry lists the block writes together
+constexpr int kHubs = 192;               // chosen nodes of a flush's pass whose long entry lists a warp each writes
+constexpr int kFlush = 4;                // nodes a thread in a flush's pass
 
 // The block's view of a launch.  Solo: this block selects for the whole level (the other blocks of the
 // cluster only help with the gain updates).
@@ -101,7 +102,7 @@ struct Shared {
     unsigned red[32];
     int2 chosen[kChosenCap];     // nodes taken and the side they move to (rebalance candidates: their gain)
     unsigned nlist, nchosen, nhub, base;
-    int2 hub[kHubs];
+    alignas(16) int4 hub[kHubs];  // node, side, first incidence, incidences
     unsigned hub_at[kHubs];
     unsigned ntie[2];
     FindScratch find;
@@ -114,6 +115,7 @@ struct Shared {
 };
 
 static_assert(offsetof(Shared, st) % 16 == 0 && offsetof(RState, hist) % 16 == 0, "the histogram is read in 16-byte pieces");
+static_assert(offsetof(Shared, hub) % 16 == 0, "16-byte entries");
 static_assert(offsetof(Shared, bits) % 16 == 0 && offsetof(LoopState, hist) == 0, "aligned");
 
 // The block's shared memory, named so that the compiler sees the address space.
@@ -227,22 +229,32 @@ __device__ __noinline__ void flush_chosen(int kind) {
         for (int i = threadIdx.x; i < n; i += kT)
             s.a.cand[s.base + i] = (unsigned long long)~gkey(s.chosen[i].y) << 32 | (unsigned)s.chosen[i].x;
     } else {
+// Bound by the chain of a node's loads, the scan and the lists' atomic: four nodes a thread share them (one a
+        // thread, and the hubs one after another with their offsets read again: 3,000 cycles for every 512 nodes,
+        // most of a selection that moves tens of thousands).
 #pragma unroll 1
-        for (int i0 = 0; i0 < n; i0 += kT) {
-            const int i = i0 + (int)threadIdx.x;
-            int v = 0, sd = 0, b = 0, d = 0, c = 0;
-            if (i < n) {
-                v = s.chosen[i].x;
-                sd = s.chosen[i].y;
-                b = __ldg(m.noff + v);
-                d = __ldg(m.noff + v + 1) - b;
-                inc += (unsigned)d;
-                const int w = __ldg(m.nw + v);
-                weight += sd ? w : -w;
-                c = d > 0 ? (int)(((unsigned)d + (unsigned)m.run - 1u) >> m.run_shift) : 1;
+        for (int i0 = 0; i0 < n; i0 += kFlush * kT) {
+            int v[kFlush], sd[kFlush], b[kFlush], d[kFlush], w[kFlush], c[kFlush], own = 0;
+#pragma unroll
+            for (int u = 0; u < kFlush; ++u) {
+                const int i = i0 + u * kT + (int)threadIdx.x;
+                const int2 x = i < n ? s.chosen[i] : make_int2(-1, 0);
+                v[u] = x.x;
+                sd[u] = x.y;
+                b[u] = v[u] >= 0 ? __ldg(m.noff + v[u]) : 0;
+                d[u] = v[u] >= 0 ? __ldg(m.noff + v[u] + 1) : 0;
+                w[u] = v[u] >= 0 ? __ldg(m.nw + v[u]) : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < kFlush; ++u) {
+                d[u] -= b[u];
+                inc += (unsigned)d[u];
+                weight += sd[u] ? w[u] : -w[u];
+                c[u] = v[u] < 0 ? 0 : (d[u] > 0 ? (int)(((unsigned)d[u] + (unsigned)m.run - 1u) >> m.run_shift) : 1);
+                own += c[u];
             }
             unsigned tot;
-            const unsigned ex = block_scan32<kT>((unsigned)c, s.red, &tot);
+            const unsigned ex = block_scan32<kT>((unsigned)own, s.red, &tot);
             if (threadIdx.x == 0) {
                 if (s.x.solo) {
                     s.base = s.rd.ents;
@@ -253,27 +265,32 @@ __device__ __noinline__ void flush_chosen(int kind) {
                 s.nhub = 0;
             }
             __syncthreads();
-            const unsigned o = s.base + ex;
-            bool mine = c > 0;
-            if (c > 8) {
-                const unsigned h = atomicAdd(&s.nhub, 1u);
-                if (h < (unsigned)kHubs) {
-                    s.hub[h] = make_int2(v, sd);
-                    s.hub_at[h] = o;
-                    mine = false;
+            unsigned o = s.base + ex;
+#pragma unroll
+            for (int u = 0; u < kFlush; ++u) {
+                bool mine = c[u] > 0;
+                if (c[u] > 8) {
+                    const unsigned h = atomicAdd(&s.nhub, 1u);
+                    if (h < (unsigned)kHubs) {
+                        s.hub[h] = make_int4(v[u], sd[u], b[u], d[u]);
+                        s.hub_at[h] = o;
+                        mine = false;
+                    }
                 }
-            }
-            if (mine)
+                if (mine)
 #pragma unroll 1
-                for (int q = 0; q < c; ++q) m.ent[o + q] = move_entry(v, b, d, q, sd, m.run);
+                    for (int q = 0; q < c[u]; ++q) m.ent[o + q] = move_entry(v[u], b[u], d[u], q, sd[u], m.run);
+                o += (unsigned)c[u];
+            }
             __syncthreads();
             const int hubs = (int)min(s.nhub, (unsigned)kHubs);
 #pragma unroll 1
-            for (int h = 0; h < hubs; ++h) {
-                const int hv = s.hub[h].x, hb = __ldg(m.noff + hv), hd = __ldg(m.noff + hv + 1) - hb;
+            for (int h = threadIdx.x >> 5; h < hubs; h += kWarps) {  // a warp each
+                const int4 hub = s.hub[h];
+                const int cnt = (int)(((unsigned)hub.w + (unsigned)m.run - 1u) >> m.run_shift);
 #pragma unroll 1
-                for (int q = threadIdx.x; q < (int)(((unsigned)hd + (unsigned)m.run - 1u) >> m.run_shift); q += kT)
-                    m.ent[s.hub_at[h] + q] = move_entry(hv, hb, hd, q, s.hub[h].y, m.run);
+                for (int q = threadIdx.x & 31; q < cnt; q += 32)
+                    m.ent[s.hub_at[h] + q] = move_entry(hub.x, hub.z, hub.w, q, hub.y, m.run);
             }
             __syncthreads();
         }
@@ -975,7 +992,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_refine_loop(const __grid_co
     }
     __syncthreads();
     const LoopArgs &a = s.a;
-    if (a.resume) {
+    const bool pend = a.resume && a.pending && __ldcg(&ls->go) != 0;
+    if (a.resume && !pend) {
         move_settle(a.m, __ldcg(&global_round()->ents), r * kT + (int)threadIdx.x, C * kT);
         if (a.solo) cluster_sync();
     }
@@ -990,7 +1008,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_refine_loop(const __grid_co
         }
     }
     int it = 0;
-    bool pending = false;   // the last selection's moves are not in the gains yet
+    bool pending = pend;    // the last selection's moves are not in the gains yet
     bool in_rebal = false;
     auto select = [&](int kind) {
         __syncthreads();
@@ -1121,6 +1139,7 @@ void launch_refine_loop(cudaStream_t s, const MoveArgs &m, const LoopParams &p, 
     a.iters = p.iters;
     a.initial = p.initial;
     a.resume = p.resume;
+    a.pending = p.pending;
     a.suspend = p.suspend;
     a.start = p.start;
     a.cmap = p.cmap;

@@ -31,6 +31,14 @@ constexpr int kLoopSoloNodes = 4096;
 // 2010, 2475; 2460 a node 2398, 1988, 2023; 4100 a node 2779, 2002, 1274; 5800 a node 3275, 1567, 1063.
 constexpr int kMoveFull = 8, kMoveFullHubs = 128, kHubDegree = 2048;
 
+// Refinement selections run on the whole grid on levels of more than kGridSelLarge nodes, and of more than
+// kGridSelNodes nodes where the coarser level has kGridSelRatio times fewer (its sides are a rough start, so many
+// nodes move); the others stay in the cluster launch, whose steps are cheaper when few do.  Bisections, cluster
+// and grid: 5M-node row-net 55.8 and 53.6 ms; 155K-node netlist merged by its largest nets (HDH, four iterations)
+// 1069 and 906 us, 600K-node row-net alike 2910 and 2658; 1M-node netlist 2753 and 2797, kept 500K-node
+// hierarchy refined 2314 and 2521.
+constexpr int kGridSelNodes = 1 << 17, kGridSelLarge = 1 << 21, kGridSelRatio = 8;
+
 // What one selection leaves for the update after it; two are used in turn.
 struct LoopRound {
     unsigned ents, items, cands, pad;
@@ -50,6 +58,9 @@ struct LoopState {
     unsigned it;       // refinement iterations done
     unsigned status0;  // the level's rebalance ran out of candidates (the last level written is 0)
     unsigned long long W[2];  // side weights
+    // a refinement selection by the grid (k_sel_count): whether it takes place, its groups' threshold gains
+    // (mode 1: all, 2: from thr up), and how many of the ties at them when not all
+    unsigned go, ticket, mode[2], thr[2], take[2];
     // a stop inside the rebalance: its state
     unsigned rebal, rounds;
     int heavy;
@@ -76,6 +87,7 @@ struct LoopParams {
     int m0, m, iters;
     bool initial;  // Algorithm 3 first (all nodes on side 1)
     bool resume;   // continue after the grid took a pending update
+    bool pending;  // resume: the grid's last selection (if it took place) is not in the gains yet
     bool suspend;  // large moves may be left to the grid
     bool start;    // the launch also projects the sides (from `coarse` by `cmap`) and counts the gains
     const int *cmap;

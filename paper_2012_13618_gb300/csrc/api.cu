@@ -647,8 +647,8 @@ void bisect_body(bipart_graph *g, Level &L0, const Params &p, int64_t W, uint8_t
     if (tail_from >= 0) {
         // the tail leaves the side of its starting level in side_a, sized for level 0 here so
         // that uncoarsen() finds it in place
-        side_buffer(g->w.side_b, std::max(L0.N, 1), g->stream);
-        uint8_t *sa = side_buffer(g->w.side_a, std::max(L0.N, 1), g->stream);
+        g->w.side_b.ensure((size_t)std::max(L0.N, 1), g->stream);
+        uint8_t *sa = (uint8_t *)g->w.side_a.ensure((size_t)std::max(L0.N, 1), g->stream);
         prof_level('t', tail_from);
         run_tail(g, levels, p, limit, W, sa);
     }
@@ -846,8 +846,8 @@ int refine_kept(bipart_graph *g, int64_t e6, int32_t iters, int *d_parts) {
     const int64_t limit[2] = {balance_limit(W, p.m0, p.m, p.e6), balance_limit(W, p.m - p.m0, p.m, p.e6)};
     uint8_t *d_side = (uint8_t *)g->side_out.ensure((size_t)L0.N, s);
     if (tail_from >= 0) {
-        side_buffer(g->w.side_b, std::max(L0.N, 1), s);
-        uint8_t *sa = side_buffer(g->w.side_a, std::max(L0.N, 1), s);
+        g->w.side_b.ensure((size_t)std::max(L0.N, 1), s);
+        uint8_t *sa = (uint8_t *)g->w.side_a.ensure((size_t)std::max(L0.N, 1), s);
         run_tail(g, levels, p, limit, W, sa);
     }
     if ((int)levels.size() != g->hier.nlev) throw Fail{BIPART_ERR_CUDA, "kept hierarchy changed size"};

@@ -38,10 +38,15 @@ void pinned_release(uint32_t *p);
 // it points to are the ones it was captured with.
 void note_realloc();
 
-// A growable device buffer (capacity only grows; contents are not preserved on growth).
+// A growable device buffer (capacity only grows; contents are not preserved on growth).  Kernels load and store
+// 16 bytes at a time and may read the last piece whole: p is 16-byte aligned whatever the allocator returned, and
+// at least 16 bytes of the allocation follow what ensure() asked for, in a reused buffer too.
 struct Buf {
+    static constexpr size_t kAlign = 16, kSlack = 16;
     void *p = nullptr;
     size_t cap = 0;
+    void *base = nullptr;  // the allocation p lies in
+    size_t size = 0;
     cudaStream_t s = nullptr;
     AllocTag tag;
     Buf() = default;
@@ -49,19 +54,22 @@ struct Buf {
     Buf &operator=(const Buf &) = delete;
     ~Buf() { release(); }
     void release() {
-        if (p) dev_free(p, cap, s, tag);
-        p = nullptr;
-        cap = 0;
+        if (base) dev_free(base, size, s, tag);
+        p = base = nullptr;
+        cap = size = 0;
     }
     void *ensure(size_t bytes, cudaStream_t stream) {
         if (bytes == 0) bytes = 16;
         if (bytes > cap) {
             release();
             s = stream;
-            size_t c = bytes + bytes / 8 + 256;
-            p = dev_alloc(c, stream, &tag);
-            if (!p) throw Fail{BIPART_ERR_OOM, "device allocation of " + std::to_string(c) + " bytes failed"};
-            cap = c;
+            const size_t c = bytes + bytes / 8 + 256;
+            base = dev_alloc(c, stream, &tag);
+            if (!base) throw Fail{BIPART_ERR_OOM, "device allocation of " + std::to_string(c) + " bytes failed"};
+            size = c;
+            const size_t shift = (0 - reinterpret_cast<uintptr_t>(base)) & (kAlign - 1);
+            p = static_cast<char *>(base) + shift;
+            cap = c - shift - kSlack;
             note_realloc();
         }
         return p;
@@ -387,8 +395,6 @@ int *degree_counters(bipart_graph *g, int32_t N);
 // the side of level tail_from in the handle's first side buffer (side_a).
 void uncoarsen(bipart_graph *g, std::vector<Level *> &levels, const int64_t limit[2], int64_t W, int m0,
                int m, int32_t iters, uint8_t *d_side0, int tail_from = -1);
-// A buffer of n sides, aligned for the four-nodes-at-a-time loads of the refinement whatever the allocator.
-uint8_t *side_buffer(Buf &b, int64_t n, cudaStream_t s);
 unsigned *bisect_status_word(bipart_graph *g);
 unsigned long long *bisect_weights(bipart_graph *g);  // the side weights of the level last refined
 // Bytes at the start of the small scratch holding counters and selection state that phases

@@ -34,11 +34,6 @@ namespace bp {
 
 namespace {
 
-template <class T>
-T *align16(T *p) {
-    return reinterpret_cast<T *>((reinterpret_cast<uintptr_t>(p) + 15) & ~uintptr_t(15));
-}
-
 constexpr int kBlock = 256;
 
 inline int grid_for(int64_t n, int per_block = kBlock, int cap = 152 * 16) {
@@ -400,8 +395,8 @@ void refine_level(bipart_graph *g, Level &L, const int *cmap, const uint8_t *coa
     m.N = L.N; m.E = L.E; m.P = L.P;
     m.noff = L.noff(); m.nadj = L.nadj(); m.hoff = L.hoff(); m.pins = L.pins(); m.hw = L.hw(); m.nw = L.nw();
     m.side = side;
-    m.prev = align16(w.side_prev.as<uint8_t>());
-    m.gain = align16(w.gain.as<int>());
+    m.prev = w.side_prev.as<uint8_t>();
+    m.gain = w.gain.as<int>();
     m.pair = w.pair.as<unsigned long long>();
     m.ls = ls;
     m.ent = w.ent.as<int4>();
@@ -497,10 +492,10 @@ void uncoarsen(bipart_graph *g, std::vector<Level *> &levels, const int64_t limi
         pmax = std::max<int64_t>(pmax, levels[l]->P);
     }
     Work &w = g->w;
-    uint8_t *sa = side_buffer(w.side_a, nmax, s);
-    uint8_t *sb = side_buffer(w.side_b, nmax, s);
-    side_buffer(w.side_prev, nmax, s);
-    w.gain.ensure(sizeof(int) * (size_t)nmax + 16, s);
+    auto *sa = (uint8_t *)w.side_a.ensure((size_t)nmax, s);
+    auto *sb = (uint8_t *)w.side_b.ensure((size_t)nmax, s);
+    w.side_prev.ensure((size_t)nmax, s);
+    w.gain.ensure(sizeof(int) * (size_t)nmax, s);
     w.pair.ensure(sizeof(unsigned long long) * (size_t)emax, s);
     static_assert(kMoveRunShort == 16 && kMoveRun == 64, "run_shift");
     // a level with short runs has at most kMoveRunShort incidences a node
@@ -527,8 +522,6 @@ void uncoarsen(bipart_graph *g, std::vector<Level *> &levels, const int64_t limi
     if (levels[0]->N > 0)
         BP_CUDA(cudaMemcpyAsync(d_side0, cur, (size_t)levels[0]->N, cudaMemcpyDeviceToDevice, s));
 }
-
-uint8_t *side_buffer(Buf &b, int64_t n, cudaStream_t s) { return align16((uint8_t *)b.ensure((size_t)n + 16, s)); }
 
 unsigned *bisect_status_word(bipart_graph *g) { return &loop_state(g)->status0; }
 

@@ -1375,6 +1375,7 @@ void run_tail(bipart_graph *g, std::vector<Level *> &levels, const Params &p, co
         for (int j = 0; j < 3 * max_new; ++j) ptrs[(size_t)j] = a.sizes + j;
         for (int j = 0; j < 3; ++j) ptrs[(size_t)3 * max_new + j] = a.info + j;
         std::vector<int32_t> v((size_t)nv);
+        const size_t recorded = g->ex.sizes.size();
         read_i32s(g, nv, ptrs.data(), v.data());
         const int nl = v[(size_t)3 * max_new];
         const int need_mb = v[(size_t)3 * max_new + 1];
@@ -1400,6 +1401,7 @@ void run_tail(bipart_graph *g, std::vector<Level *> &levels, const Params &p, co
         }
         if (need_mb > 0) {
             if (g->ex.capturing || attempt > 8) throw Fail{BIPART_ERR_OOM, "tail arena too small"};
+            if (g->ex.recording) g->ex.sizes.resize(recorded);  // only the run that fits is captured later
             w.t_arena.ensure(std::max<size_t>(2 * w.t_arena.cap, ((size_t)need_mb << 20) * 2), s);
             continue;
         }

@@ -697,15 +697,13 @@ bool coarsen_level(bipart_graph *g, Level &f, Level &c, int policy, int32_t *siz
 }
 
 void coarsen_init() {
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, []() {
+    static PerDevice set;
+    set.get([]() {
         const int bytes = (int)(sizeof(int) * kPrivNodesWide);
-        err = cudaFuncSetAttribute(k_seg_copy_priv, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (err == cudaSuccess)
-            err = cudaFuncSetAttribute(k_fill_adj_priv, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        BP_CUDA(cudaFuncSetAttribute(k_seg_copy_priv, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        BP_CUDA(cudaFuncSetAttribute(k_fill_adj_priv, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        return 1;
     });
-    BP_CUDA(err);
 }
 
 }  // namespace bp

@@ -7,6 +7,7 @@
 
 #include <condition_variable>
 #include <functional>
+#include <map>
 #include <memory>
 #include <mutex>
 #include <string>
@@ -37,6 +38,24 @@ void pinned_release(uint32_t *p);
 // Bumped whenever a buffer is (re)allocated: a captured graph is only valid while the buffers
 // it points to are the ones it was captured with.
 void note_realloc();
+
+// A value made once for every device a process uses, under a lock (the attributes of a kernel belong to one device).
+class PerDevice {
+   public:
+    template <class Make>
+    int get(Make make) {
+        int dev = 0;
+        BP_CUDA(cudaGetDevice(&dev));
+        std::lock_guard<std::mutex> lk(mu_);
+        auto it = value_.find(dev);
+        if (it == value_.end()) it = value_.emplace(dev, make()).first;
+        return it->second;
+    }
+
+   private:
+    std::mutex mu_;
+    std::map<int, int> value_;
+};
 
 // A growable device buffer (capacity only grows; contents are not preserved on growth).  Kernels load and store
 // 16 bytes at a time and may read the last piece whole: p is 16-byte aligned whatever the allocator returned, and
@@ -400,7 +419,7 @@ unsigned long long *bisect_weights(bipart_graph *g);  // the side weights of the
 // Bytes at the start of the small scratch holding counters and selection state that phases
 // leave zero for the next one (cleared once at the start of every bisection).
 size_t small_state_bytes();
-void refine_init();  // once per process: kernel attributes (never during a capture)
+void refine_init();  // once per device: kernel attributes (never during a capture)
 void coarsen_init();  // same, for the coarsening kernels
 // Weight limit of a side meant for ms of m parts of a (sub)graph of weight W, imbalance e6
 // millionths: max(ceil(W ms / m), floor(W ms (10^6 + e6) / (m 10^6))) (reading C12; G2 for

@@ -24,7 +24,6 @@
 #include <algorithm>
 #include <climits>
 #include <cstddef>
-#include <mutex>
 
 #include <cooperative_groups.h>
 #include <cooperative_groups/scan.h>
@@ -1079,8 +1078,6 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_refine_loop(const __grid_co
 
 // ------------------------------------------------------------------------ host side
 namespace {
-std::once_flag g_loop_once;
-int g_loop_cluster = 0;
 constexpr size_t kLoopKeys = sizeof(Shared) - offsetof(Shared, bits);  // bytes the sort keys have without asking
 
 // Dynamic shared memory of a launch whose rebalance sorts up to sq keys.
@@ -1091,9 +1088,10 @@ size_t loop_smem(int64_t sq) {
 }
 }  // namespace
 
-// Largest cluster of k_refine_loop this GPU runs (1 always works).
+// Largest cluster of k_refine_loop the current device runs (1 always works).
 static int loop_cluster() {
-    std::call_once(g_loop_once, []() {
+    static PerDevice cluster;
+    return cluster.get([]() {
         BP_CUDA(cudaFuncSetAttribute(k_refine_loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)loop_smem(kRebalMax)));
         BP_CUDA(cudaFuncSetAttribute(k_refine_loop, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
@@ -1110,15 +1108,11 @@ static int loop_cluster() {
             cfg.attrs = at;
             cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, k_refine_loop, &cfg) == cudaSuccess && n >= 1) {
-                g_loop_cluster = c;
-                break;
-            }
+            if (cudaOccupancyMaxActiveClusters(&n, k_refine_loop, &cfg) == cudaSuccess && n >= 1) return c;
             cudaGetLastError();
         }
-        if (g_loop_cluster == 0) throw Fail{BIPART_ERR_CUDA, "the refinement kernel does not fit this GPU"};
+        throw Fail{BIPART_ERR_CUDA, "the refinement kernel does not fit this GPU"};
     });
-    return g_loop_cluster;
 }
 
 void refine_init() { loop_cluster(); }

@@ -41,7 +41,6 @@
 #include <cstddef>
 #include <cstdio>
 #include <cstdlib>
-#include <mutex>
 
 #include <cooperative_groups.h>
 
@@ -1244,21 +1243,29 @@ __global__ void __launch_bounds__(kTT, 1) k_tail(TailArgs a) {
 
 // ------------------------------------------------------------------ host side
 namespace {
-std::once_flag g_tail_once;
-int g_tail_cluster = 0;      // blocks per cluster (0: the tail is not used)
-int g_tail_nodes = kTailNodes;
-int64_t g_tail_pins = kTailStartPins;
+// Where the tail may start (BIPART_TAIL_NODES and BIPART_TAIL_PINS, read once, lower or raise the limits).
+struct TailLimits {
+    int nodes = kTailNodes;
+    int64_t pins = kTailStartPins;
+    TailLimits() {
+        if (const char *env = std::getenv("BIPART_TAIL_NODES")) nodes = std::min(std::atoi(env), kTailNodes);
+        if (const char *env = std::getenv("BIPART_TAIL_PINS")) pins = std::min<int64_t>(std::atoll(env), kTailMaxPins);
+    }
+};
+const TailLimits &tail_limits() {
+    static const TailLimits limits;
+    return limits;
+}
 }  // namespace
 
 int tail_cluster() {
-    std::call_once(g_tail_once, []() {
-        if (const char *env = std::getenv("BIPART_TAIL_NODES")) g_tail_nodes = std::min(std::atoi(env), kTailNodes);
-        if (const char *env = std::getenv("BIPART_TAIL_PINS")) g_tail_pins = std::min<int64_t>(std::atoll(env), kTailMaxPins);
-        if (g_tail_nodes <= 0) return;
+    static PerDevice cluster;
+    if (tail_limits().nodes <= 0) return 0;
+    return cluster.get([]() {
         if (cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) != cudaSuccess ||
             cudaFuncSetAttribute(k_tail, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
             cudaGetLastError();
-            return;
+            return 0;
         }
         for (int c : {16, 8, 4}) {
             cudaLaunchConfig_t cfg = {};
@@ -1273,22 +1280,19 @@ int tail_cluster() {
             cfg.attrs = at;
             cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, k_tail, &cfg) == cudaSuccess && n >= 1) {
-                g_tail_cluster = c;
-                break;
-            }
+            if (cudaOccupancyMaxActiveClusters(&n, k_tail, &cfg) == cudaSuccess && n >= 1) return c;
             cudaGetLastError();
         }
+        return 0;
     });
-    return g_tail_cluster;
 }
 
 bool tail_eligible(const Level &L, int max_new, int flags) {
-    const int C = tail_cluster();  // first: it also reads the limits' overrides
+    const int C = tail_cluster();
     if (C <= 0) return false;
     if (flags & BIPART_FLAG_MERGE_PARALLEL) return false;  // the tail runs the paper's contraction
     if (max_new > kTailMaxLevels || L.N < 1) return false;
-    if (L.N > g_tail_nodes || (int64_t)L.P > g_tail_pins) return false;
+    if (L.N > tail_limits().nodes || (int64_t)L.P > tail_limits().pins) return false;
     // every block's share of the chunk table fits its shared-memory copy
     return (tail_chunks(L.P) + C - 1) / C + 1 <= kTailMaxChunks;
 }

@@ -188,14 +188,13 @@ struct Work {
     Buf small;       // small device scalars (counters, totals, selection state)
     Buf e_a, e_b, e_c, e_d;  // per-hyperedge int32 scratch
     Buf e_key;       // per-hyperedge uint64 keys
-    Buf n_a, n_b, n_c;       // per-node int32 scratch
-    Buf n_key;       // per-node uint64 keys
+    Buf n_a, n_b;    // per-node int32 scratch
+    Buf n_c;         // per-node int32 scratch; refinement: gains
+    Buf n_key;       // per-node uint64 keys; refinement: moved nodes' incidence runs
     Buf p_a;         // per-pin int32 scratch
     Buf side_a, side_b;      // uint8 sides (ping-pong across levels)
-    Buf gain;        // int32 gains
     Buf side_prev;   // uint8 sides before the last selection
     Buf pair;        // uint64 pins on side 0 << 32 | pins on side 1 of every hyperedge
-    Buf ent;         // moved nodes' incidence runs
     Buf items;       // work items of wide hyperedges whose contributions changed
     Buf e_best;      // per-hyperedge uint64 singleton-attach keys
     Buf m_fp, m_tkey, m_tmin, m_rep, m_wsum;  // parallel-net merging: fingerprints, table, groups

@@ -9,7 +9,7 @@
 //
 // Scratch: g_cut_scratch holds, per call, a small header (completion counter, error flag, list length),
 // the per-block partial sums and the list of the hyperedges that take a block each.  It is sized
-// for at most kCutNoAllocMaxHedges hyperedges (16 MiB plus 33 KiB on every GPU that loads the
+// for at most kCutNoAllocMaxHedges hyperedges (16 MiB plus 15 KiB on every GPU that loads the
 // library, held until the process exits).  Every call uses the same array: calls that overlap
 // on the GPU (different streams, or different host threads on the same device) race on it and
 // must be serialised by the caller.

@@ -384,6 +384,9 @@ LoopState *loop_state(bipart_graph *g) {
     return reinterpret_cast<LoopState *>(g->w.small.as<char>() + 256);
 }
 
+// Nodes with short incidence lists share a warp four at a time.
+bool short_lists(const Level &L) { return (int64_t)L.P <= kMoveRunShort * (int64_t)L.N; }
+
 // A level's refinement from the sides in `side` (k_level_start projects them from `coarse`, the
 // sides of the next coarser level; null: the coarsest level, with Algorithm 3 first).
 void refine_level(bipart_graph *g, Level &L, const int *cmap, const uint8_t *coarse, int coarse_n, uint8_t *side,
@@ -396,17 +399,16 @@ void refine_level(bipart_graph *g, Level &L, const int *cmap, const uint8_t *coa
     m.noff = L.noff(); m.nadj = L.nadj(); m.hoff = L.hoff(); m.pins = L.pins(); m.hw = L.hw(); m.nw = L.nw();
     m.side = side;
     m.prev = w.side_prev.as<uint8_t>();
-    m.gain = w.gain.as<int>();
+    m.gain = w.n_c.as<int>();
     m.pair = w.pair.as<unsigned long long>();
     m.ls = ls;
-    m.ent = w.ent.as<int4>();
+    m.ent = w.n_key.as<int4>();
     m.items = w.items.as<int4>();
     m.item_cap = kItemCap;
-    // nodes with short incidence lists share a warp four at a time
-    const bool short_lists = (int64_t)L.P <= kMoveRunShort * (int64_t)L.N;
-    m.lanes = short_lists ? 8 : 32;
-    m.run = short_lists ? kMoveRunShort : kMoveRun;
-    m.run_shift = short_lists ? 4 : 6;
+    const bool shorter = short_lists(L);
+    m.lanes = shorter ? 8 : 32;
+    m.run = shorter ? kMoveRunShort : kMoveRun;
+    m.run_shift = shorter ? 4 : 6;
     p.sq = ceil_sqrt64(L.N);
     if (p.sq > kRebalMax) throw Fail{BIPART_ERR_OOM, "level too large for the ordered rebalance"};
     auto *cand = (unsigned long long *)w.list.ensure(sizeof(unsigned long long) * (size_t)std::max<int64_t>(p.sq, 1), s);
@@ -485,21 +487,24 @@ void uncoarsen(bipart_graph *g, std::vector<Level *> &levels, const int64_t limi
     cudaStream_t s = g->stream;
     const int Lc = (int)levels.size() - 1;
     const int top = tail_from >= 0 ? tail_from : Lc;  // the coarsest level refined on the grid
-    int64_t nmax = 1, emax = 1, pmax = 1;
+    int64_t nmax = 1, emax = 1, ents = 1;
     for (int l = 0; l <= top; ++l) {
-        nmax = std::max<int64_t>(nmax, levels[l]->N);
-        emax = std::max<int64_t>(emax, levels[l]->E);
-        pmax = std::max<int64_t>(pmax, levels[l]->P);
+        const Level &L = *levels[l];
+        nmax = std::max<int64_t>(nmax, L.N);
+        emax = std::max<int64_t>(emax, L.E);
+        // a node of d incidences takes max(1, ceil(d / run)) <= 1 + d / run entries of the move list
+        ents = std::max<int64_t>(ents, L.N + (int64_t)L.P / (short_lists(L) ? kMoveRunShort : kMoveRun));
     }
     Work &w = g->w;
     auto *sa = (uint8_t *)w.side_a.ensure((size_t)nmax, s);
     auto *sb = (uint8_t *)w.side_b.ensure((size_t)nmax, s);
     w.side_prev.ensure((size_t)nmax, s);
-    w.gain.ensure(sizeof(int) * (size_t)nmax, s);
+    // the coarsening's scratch of the same handle is free by now: at many nodes and few pins these two would be a
+    // third of a request's memory
+    w.n_c.ensure(sizeof(int) * (size_t)nmax, s);
+    w.n_key.ensure(sizeof(int4) * (size_t)ents, s);
     w.pair.ensure(sizeof(unsigned long long) * (size_t)emax, s);
     static_assert(kMoveRunShort == 16 && kMoveRun == 64, "run_shift");
-    // a level with short runs has at most kMoveRunShort incidences a node
-    w.ent.ensure(sizeof(int4) * (size_t)(nmax + std::max<int64_t>(pmax / kMoveRun, nmax) + 1), s);
     w.items.ensure(sizeof(int4) * (size_t)kItemCap, s);
 
     LoopParams p{};

@@ -160,14 +160,6 @@ struct TLev {
 // Slice of [0, n) owned by block r of C.
 __device__ __forceinline__ int slice_lo(int n, int r, int C) { return (int)((long long)n * r / C); }
 
-// The block whose slice holds node v.
-__device__ __forceinline__ int slice_of(int n, int v, int C) {
-    int q = (int)((long long)v * C / n);
-    while (q > 0 && v < slice_lo(n, q, C)) --q;
-    while (q + 1 < C && v >= slice_lo(n, q + 1, C)) ++q;
-    return q;
-}
-
 // Chunk table entries of hyperedge e (first pin o, k pins): every boundary c * kQ in (o, o + k]
 // starts its chunk at hyperedge e + 1 (pin o + k).
 __device__ __forceinline__ void mark_chunks(int *ce, int *cp, int e, int o, int k) {

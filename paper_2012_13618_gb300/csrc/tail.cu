@@ -60,7 +60,12 @@ namespace {
 constexpr int kTT = kTailThreads;
 constexpr int kNT = kTailNodes;
 constexpr int kQ = kTailChunk;
-constexpr int kThreadPins = 32; // refinement: hyperedges up to this degree: one thread; above: one warp
+// Refinement: hyperedges of up to kThreadPins pins take a thread, up to kGroupPins eight lanes, wider ones a warp;
+// of a level whose pins are read through L2 up to kGroupPins a thread, wider ones a warp.  With up to 32 pins a
+// thread the longest loop was the pass (row-net level of 966 nodes, 20K pins: gains 26 us a pass, now 10, weighted
+// degrees 18 and 7; replays of row-nets of 2,000-8,000 nodes 1.1-1.4 times as long as on the grid, now 0.75-1.05);
+// all warps on the hyperedges of more than 256 pins gave nothing.
+constexpr int kThreadPins = 8, kGroupPins = 32;
 constexpr int kThreadDeg = 16;  // hyperedges up to this degree: one thread; above: one warp
 constexpr int kWarpDeg = 256;   // contraction: above this, the whole block (bitmap)
 
@@ -99,8 +104,9 @@ constexpr size_t kSmemMax = 216 * 1024;  // with the kernel's static arrays (9.6
 struct TinyLevel {
     int N, E, P;
     const int *hoff, *pins, *hw;
-    int gain, deg, nw, wide, sp, so;  // offsets: gains, weighted degrees, weights; wide hyperedges, 16-bit pins
-    bool staged;                      // and offsets, when the hyperedges are staged
+    int gain, deg, nw, list, sp, so;  // offsets: gains, weighted degrees, weights; 16-bit lists of hyperedges, pins
+    int list_cap;                     // and offsets, when the hyperedges are staged
+    bool staged;
 };
 
 // Shared memory of the refinement: this, then the level's node arrays and its staged hyperedges.
@@ -110,7 +116,7 @@ struct Tiny {
     FindScratch find;
     CutScratch cut;
     unsigned red[32];
-    unsigned ncand, nwide;
+    unsigned ncand, ngroup, nwide;
     int wdelta;                                // weight moved to side 1 less that moved to side 0
     unsigned long long keys[kRebalKeys];       // the rebalance's candidates: gain descending << 32 | node
     unsigned tie[2][kTieWords], pre[kTieWords];
@@ -745,20 +751,22 @@ struct GlobalPins {
 __device__ __noinline__ void tiny_load(const TLev &L) {
     Tiny &s = tiny();
     const int n4 = 4 * ((L.N + 3) & ~3);
-    const int wide_cap = L.P / (kThreadPins + 1) + 1;
     TinyLevel t;
     t.N = L.N; t.E = L.E; t.P = L.P;
     t.hoff = L.hoff; t.pins = L.pins; t.hw = L.hw;
     t.gain = (int)kTinyFixed;
     t.deg = t.gain + n4;
     t.nw = t.deg + n4;
-    t.wide = t.nw + n4;
-    t.sp = (t.wide + 4 * wide_cap + 7) & ~7;
+    // hyperedges of more than kThreadPins pins: those of a group of lanes from the front, of a warp from the back
+    t.list = t.nw + n4;
+    t.list_cap = L.P / (kThreadPins + 1) + 1;
+    t.sp = (t.list + 2 * t.list_cap + 7) & ~7;
     t.so = t.sp + 2 * ((L.P + 3) & ~3);
-    t.staged = L.P < 65536 && kTinyFixed + 3 * (size_t)n4 + 4 * (size_t)wide_cap + 16 + 2 * (size_t)L.P + 2 * (size_t)L.E <= kSmemMax;
+    t.staged = L.P < 65536 && L.E < 65536 &&
+               kTinyFixed + 3 * (size_t)n4 + 2 * (size_t)t.list_cap + 16 + 2 * (size_t)L.P + 2 * (size_t)L.E <= kSmemMax;
     if (threadIdx.x == 0) {
         s.lev = t;
-        s.nwide = 0;
+        s.ngroup = s.nwide = 0;
     }
     __syncthreads();
 #pragma unroll 1
@@ -768,6 +776,7 @@ __device__ __noinline__ void tiny_load(const TLev &L) {
     }
     if (t.staged) {
         uint16_t *sp = reinterpret_cast<uint16_t *>(tiny_at(t.sp)), *so = reinterpret_cast<uint16_t *>(tiny_at(t.so));
+        uint16_t *list = reinterpret_cast<uint16_t *>(tiny_at(t.list));
         const bool vec = (reinterpret_cast<uintptr_t>(L.pins) & 15) == 0;
         const int quads = vec ? L.P >> 2 : 0;
 #pragma unroll 1
@@ -798,7 +807,9 @@ __device__ __noinline__ void tiny_load(const TLev &L) {
                 const int e = e0 + k * kTT;
                 if (e >= L.E) continue;
                 so[e] = (uint16_t)o[k];
-                if (q[k] - o[k] > kThreadPins) tiny_ints(t.wide)[atomicAdd(&s.nwide, 1u)] = e;
+                const int d = q[k] - o[k];
+                if (d > kGroupPins) list[t.list_cap - 1 - (int)atomicAdd(&s.nwide, 1u)] = (uint16_t)e;
+                else if (d > kThreadPins) list[atomicAdd(&s.ngroup, 1u)] = (uint16_t)e;
             }
         }
         if (threadIdx.x == 0) so[L.E] = (uint16_t)L.P;
@@ -813,21 +824,45 @@ __device__ __forceinline__ void tiny_wide(Pins pin, const int *hw, const uint8_t
     const int lane = threadIdx.x & 31;
     int n1 = 0;
     if (gains) {
-#pragma unroll 2
+#pragma unroll 4
         for (int i = lane; i < d; i += 32) n1 += side[pin(b + i)];
         n1 = __reduce_add_sync(0xffffffffu, n1);
         if (n1 == 0 || n1 == d) return;
     }
     const int w = hw ? __ldcg(hw + e) : 1;
     const int x1 = n1 == 1 ? 2 * w : w, x0 = gains && d - n1 == 1 ? 2 * w : w;
-#pragma unroll 2
+#pragma unroll 4
     for (int i = lane; i < d; i += 32) {
         const int u = pin(b + i);
         atomicAdd(out + u, gains && side[u] ? x1 : x0);
     }
 }
 
-// K hyperedges of up to kThreadPins pins by a thread (d[k] = 0: none).  The first four pins of all of them are
+// A listed hyperedge by eight lanes, four at most of a warp at once (d = 0: none); all lanes of the warp.
+template <class Pins>
+__device__ __forceinline__ void tiny_group(Pins pin, const int *hw, const uint8_t *side, int *out, bool gains, int e,
+                                           int b, int d) {
+    const int sub = threadIdx.x & 7;
+    int u[kGroupPins / 8], n1 = 0;
+    unsigned on1 = 0;
+#pragma unroll
+    for (int k = 0; k < kGroupPins / 8; ++k) u[k] = sub + 8 * k < d ? pin(b + sub + 8 * k) : 0;
+    if (gains) {
+#pragma unroll
+        for (int k = 0; k < kGroupPins / 8; ++k) on1 |= (sub + 8 * k < d ? (unsigned)side[u[k]] : 0u) << k;
+        n1 = __popc(on1);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) n1 += __shfl_xor_sync(0xffffffffu, n1, o);
+        if (n1 == 0 || n1 == d) return;
+    }
+    const int w = hw && d > 0 ? __ldcg(hw + e) : 1;
+    const int x1 = n1 == 1 ? 2 * w : w, x0 = gains && d - n1 == 1 ? 2 * w : w;
+#pragma unroll
+    for (int k = 0; k < kGroupPins / 8; ++k)
+        if (sub + 8 * k < d) atomicAdd(out + u[k], on1 >> k & 1u ? x1 : x0);
+}
+
+// K hyperedges by a thread (d[k] = 0: none).  The first four pins of all of them are
 // handled straight-line, predicated: a loop per hyperedge costs a chain of shared-memory latencies and a
 // divergence each.
 template <int K, class Pins>
@@ -867,8 +902,7 @@ __device__ __forceinline__ void tiny_some(Pins pin, const int *hw, const uint8_t
 }
 
 // A pass over the level's hyperedges.  With `sides` (offset of the sides): Algorithm 4's gains, the cut
-// hyperedges' contributions added to the gains; without (-1): the weighted degrees.  Hyperedges of up to
-// kThreadPins pins take a thread, wider ones a warp.
+// hyperedges' contributions added to the gains; without (-1): the weighted degrees.
 __device__ __noinline__ void tiny_edges(int sides) {
     Tiny &s = tiny();
     const int lane = threadIdx.x & 31, E = s.lev.E;
@@ -893,10 +927,19 @@ __device__ __noinline__ void tiny_edges(int sides) {
             tiny_some<K>(pin, hw, side, out, gains, e, b, d);
         }
         __syncwarp();
+        const uint16_t *list = reinterpret_cast<const uint16_t *>(tiny_at(s.lev.list));
+        const int ngroup = (int)s.ngroup, nwide = (int)s.nwide, cap = s.lev.list_cap;
 #pragma unroll 1
-        for (int i = threadIdx.x >> 5; i < (int)s.nwide; i += kTT / 32) {
-            const int e = tiny_ints(s.lev.wide)[i];
+        for (int i = threadIdx.x >> 5; i < nwide; i += kTT / 32) {
+            const int e = list[cap - 1 - i];
             tiny_wide(pin, hw, side, out, gains, e, so[e], so[e + 1] - so[e]);
+            __syncwarp();
+        }
+#pragma unroll 1
+        for (int i0 = 4 * (int)(threadIdx.x >> 5); i0 < ngroup; i0 += 4 * (kTT / 32)) {
+            const int i = i0 + (lane >> 3), e = i < ngroup ? list[i] : 0, b = so[e];
+            tiny_group(pin, hw, side, out, gains, e, b, i < ngroup ? so[e + 1] - b : 0);
+            __syncwarp();
         }
     } else {
         const GlobalPins pin{s.lev.pins};
@@ -913,8 +956,8 @@ __device__ __noinline__ void tiny_edges(int sides) {
             }
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                todo[k] = __ballot_sync(0xffffffffu, d[k] > kThreadPins);
-                f[k] = d[k] > kThreadPins ? 0 : d[k];
+                todo[k] = __ballot_sync(0xffffffffu, d[k] > kGroupPins);
+                f[k] = d[k] > kGroupPins ? 0 : d[k];
             }
             tiny_some<K>(pin, hw, side, out, gains, e, b, f);
             __syncwarp();

@@ -722,26 +722,15 @@ __device__ __noinline__ void select_nodes(int kind) {
     sel_sync();
 }
 
-// The level's sides, pairs and gains (what k_level_start, k_hedge_n1 and k_node_gain do on large levels), by
-// all blocks, hyperedge by hyperedge: its side-1 pins counted, its pair stored, its contributions added to
-// its pins' gains.  Up to 32 pins take one thread, more a warp.  Levels whose nodes have many incidences add
+// The level's pairs and gains counted from the sides (what k_hedge_n1 and k_node_gain do on large levels), by all
+// blocks, hyperedge by hyperedge: its side-1 pins counted, its pair stored, its contributions added to its pins'
+// gains, which are zero.  Up to 32 pins take one thread, more a warp.  Levels whose nodes have many incidences add
 // up in shared memory first: few nodes would take many atomics each.
-__device__ __noinline__ void start_level() {
+__device__ __noinline__ void count_level() {
     Shared &s = sh();
     const Ctx &x = s.x;
-    const LoopArgs &a = s.a;
-    const MoveArgs &m = a.m;
+    const MoveArgs &m = s.a.m;
     const int rank = x.r * kT + (int)threadIdx.x, size = x.C * kT, lane = threadIdx.x & 31;
-#pragma unroll 1
-    for (int v = rank; v < m.N; v += size) {
-        const uint8_t sd = a.cmap ? __ldg(a.coarse + __ldg(a.cmap + v)) : (uint8_t)1;
-        m.side[v] = sd;
-        m.prev[v] = sd;
-        m.gain[v] = 0;
-    }
-    if (x.r == x.C - 1)
-        for (int i = threadIdx.x; i < (int)(offsetof(LoopState, cmd) / sizeof(unsigned)); i += kT)
-            reinterpret_cast<unsigned *>(m.ls)[i] = 0;
     constexpr int kAcc = (int)(sizeof(s.chosen) / sizeof(int));
     int *acc = reinterpret_cast<int *>(sh().chosen);
     const bool priv = m.N <= kAcc && m.P > 8 * m.N;
@@ -803,6 +792,24 @@ __device__ __noinline__ void start_level() {
     cluster_sync();
 }
 
+// The level's sides projected and everything counted, by all blocks (small levels).
+__device__ __noinline__ void start_level() {
+    const LoopArgs &a = sh().a;
+    const MoveArgs &m = a.m;
+    const int r = sh().x.r, C = sh().x.C;
+#pragma unroll 1
+    for (int v = r * kT + (int)threadIdx.x; v < m.N; v += C * kT) {
+        const uint8_t sd = a.cmap ? __ldg(a.coarse + __ldg(a.cmap + v)) : (uint8_t)1;
+        m.side[v] = sd;
+        m.prev[v] = sd;
+        m.gain[v] = 0;
+    }
+    if (r == C - 1)
+        for (int i = threadIdx.x; i < (int)(offsetof(LoopState, cmd) / sizeof(unsigned)); i += kT)
+            reinterpret_cast<unsigned *>(m.ls)[i] = 0;
+    count_level();
+}
+
 // Gains after the last selection's moves, by all blocks.  own: exact for the moved nodes too (a
 // rebalance leaves them out: they are on the light side, which stays the light side until the
 // level is done).
@@ -832,12 +839,14 @@ __device__ __noinline__ void update_gains(bool own) {
         if (tid == 0) {
             ls->rd[0].ents = n;
             ls->rd[0].items = 0;
+            ls->rd[0].inc = s.rd.inc;
             ls->cmd = 1u | (unsigned)own << 1;
         }
         cluster_sync();  // the helpers read the command after this barrier
     } else {
         n = __ldcg(&ls->rd[x.p].ents);
     }
+    const bool full = (long long)__ldcg(&ls->rd[x.solo ? 0 : x.p].inc) * kMoveCount > (long long)m.P;
     LoopRound *rd = &ls->rd[x.solo ? 0 : x.p];
     // the histogram and the other round's lists are clear for the next selection
     if (!x.solo && x.r == x.C - 1) {
@@ -845,14 +854,19 @@ __device__ __noinline__ void update_gains(bool own) {
         unsigned *other = reinterpret_cast<unsigned *>(&ls->rd[x.p ^ 1]);
         for (int i = tid; i < (int)(sizeof(LoopRound) / sizeof(unsigned)); i += kT) other[i] = 0;
     }
-    // a warp per entry, the blocks' first warps first: a short list spreads over all SMs
-    const int warp = (tid >> 5) * x.C + x.r, warps = x.C * kWarps;
-    move_pass1(m, n, &rd->items, warp, warps, wside, false);
-    cluster_sync();
-    const unsigned items = __ldcg(&rd->items);
-    if (own || items > 0) {
-        move_pass2(m, n, items, warp, warps, wside, own);
+    if (full) {
+        for (int v = x.r * kT + tid; v < m.N; v += x.C * kT) m.gain[v] = 0;
+        count_level();
+    } else {
+        // a warp per entry, the blocks' first warps first: a short list spreads over all SMs
+        const int warp = (tid >> 5) * x.C + x.r, warps = x.C * kWarps;
+        move_pass1(m, n, &rd->items, warp, warps, wside, false);
         cluster_sync();
+        const unsigned items = __ldcg(&rd->items);
+        if (own || items > 0) {
+            move_pass2(m, n, items, warp, warps, wside, own);
+            cluster_sync();
+        }
     }
     if (x.solo) {
         if (x.r != 0) return;

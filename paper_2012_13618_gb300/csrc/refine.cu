@@ -413,7 +413,7 @@ void refine_level(bipart_graph *g, Level &L, const int *cmap, const uint8_t *coa
     if (p.sq > kRebalMax) throw Fail{BIPART_ERR_OOM, "level too large for the ordered rebalance"};
     auto *cand = (unsigned long long *)w.list.ensure(sizeof(unsigned long long) * (size_t)std::max<int64_t>(p.sq, 1), s);
     const bool warp_sum = (int64_t)L.P > kWarpSumDegree * (int64_t)L.N;
-    p.start = L.P <= kLoopStartPins;
+    p.start = L.P <= kLoopStartPins && L.N <= kLoopStartNodes;
     p.cmap = cmap;
     p.coarse = coarse;
     if (!p.start) {
@@ -423,19 +423,21 @@ void refine_level(bipart_graph *g, Level &L, const int *cmap, const uint8_t *coa
                                                                           m.gain, m.hoff, m.pair, ls);
             BP_LAUNCH();
         }
-        {
+        if (L.P > 0) {
             // hoff, pins, one side byte per pin, one atomic per hyperedge run
             ProfScope ps("hedge_n1", 8.0 * L.E + 5.0 * L.P, s);
             k_hedge_n1<<<lb_grid(L.P), kLbBlock, 0, s>>>(L.E, L.P, L.hoff(), L.pins(), side, m.pair, L.tsh());
             BP_LAUNCH();
         }
-        // noff, nadj, 8-byte pair gather per incidence (and a weight where it counts), side, gain
-        ProfScope ps("node_gain", 9.0 * L.N + 12.0 * L.P, s);
-        k_node_gain<<<lb_grid(L.P), kLbBlock, 0, s>>>(L.N, L.P, L.noff(), L.nadj(), m.pair, L.hw(), side, m.gain,
-                                                       L.tsn(), warp_sum);
-        BP_LAUNCH();
+        if (L.P > 0) {
+            // noff, nadj, 8-byte pair gather per incidence (and a weight where it counts), side, gain
+            ProfScope ps("node_gain", 9.0 * L.N + 12.0 * L.P, s);
+            k_node_gain<<<lb_grid(L.P), kLbBlock, 0, s>>>(L.N, L.P, L.noff(), L.nadj(), m.pair, L.hw(), side, m.gain,
+                                                           L.tsn(), warp_sum);
+            BP_LAUNCH();
+        }
     }
-    p.suspend = L.P > kLoopAlonePins;
+    p.suspend = L.P > kLoopAlonePins || L.N > kGridSelLarge;
     p.resume = false;
     if (p.suspend && !p.initial && (L.N > kGridSelLarge || (L.N > kGridSelNodes && L.N / kGridSelRatio >= coarse_n))) {
         auto *ties = reinterpret_cast<unsigned *>(cand);  // the rebalance's candidates come later

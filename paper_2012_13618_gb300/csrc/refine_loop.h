@@ -20,8 +20,9 @@ constexpr int kItemCap = 1 << 16;       // work items a pass may queue (beyond: 
 // the one cluster (levels of more than kLoopAlonePins pins only; smaller ones stay in the cluster).
 constexpr long long kLoopMoveInc = 1 << 17;
 constexpr int64_t kLoopAlonePins = 1 << 18;
-// Levels of at most this many pins are started (sides projected, gains counted) by the cluster launch too.
-constexpr int kLoopStartPins = 1 << 17;
+// Levels of at most this many pins are started (sides projected, gains counted) by the cluster launch too, unless they
+// have more nodes than kLoopStartNodes: its 8,192 threads project a node each at a time.
+constexpr int kLoopStartPins = 1 << 17, kLoopStartNodes = 1 << 16;
 // Levels of at most this many nodes are selected by the cluster's first block alone, the others helping
 // with the gain updates only.
 constexpr int kLoopSoloNodes = 4096;
@@ -37,7 +38,7 @@ constexpr int kMoveFull = 8, kMoveFullHubs = 128, kHubDegree = 2048;
 constexpr int kMoveCount = 8;
 
 // Refinement selections run on the whole grid on levels of more than kGridSelLarge nodes, and of more than
-// kGridSelNodes nodes where the coarser level has kGridSelRatio times fewer (its sides are a rough start, so many
+// kGridSelNodes nodes and kLoopAlonePins pins where the coarser level has kGridSelRatio times fewer (its sides are a rough start, so many
 // nodes move); the others stay in the cluster launch, whose steps are cheaper when few do.  Bisections, cluster
 // and grid: 5M-node row-net 55.8 and 53.6 ms; 155K-node netlist merged by its largest nets (HDH, four iterations)
 // 1069 and 906 us, 600K-node row-net alike 2910 and 2658; 1M-node netlist 2753 and 2797, kept 500K-node

@@ -562,7 +562,6 @@ void extract_subgraph(bipart_graph *g, const int *d_part, int j, bipart_graph *k
         S.E = E;
         S.P = P;
         S.unit_hw = L.unit_hw;
-        S.wide = L.wide;
         kid->l2g.ensure(sizeof(int) * (size_t)std::max(N, 1), ks);
         S.b_nw.ensure(sizeof(int) * (size_t)std::max(N, 1), ks);
         S.b_hoff.ensure(sizeof(int) * ((size_t)E + 1), ks);

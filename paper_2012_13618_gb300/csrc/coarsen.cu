@@ -504,12 +504,11 @@ void contract(bipart_graph *g, int32_t E, int32_t P, const int *hoff, const int 
             ProfScope ps("contract_offsets", 16.0 * E, s);
             scan(E, CompactIn{cnt, rep}, out, w.scan, dev_status(g), s);
         }
-        // n_slot lies before sizes, and for level 0 the length of the list of wide hyperedges: one copy
-        const int32_t *ptr[3] = {n_slot ? n_slot : small + 1, sizes, sizes + 1};
+        const int32_t *ptr[3] = {n_slot, sizes, sizes + 1};  // n_slot lies before sizes: one copy
         int32_t v[3];
-        read_i32s(g, 3, ptr, v);
+        const int first = n_slot ? 0 : 1;
+        read_i32s(g, 3 - first, ptr + first, v + first);
         if (n_slot) c.N = v[0];
-        else if (!map) c.wide = v[0] > 0;
         c.E = v[1];
         c.P = v[2];
         {
@@ -528,7 +527,6 @@ void contract(bipart_graph *g, int32_t E, int32_t P, const int *hoff, const int 
         c.E = 0;
         c.P = 0;
         if (n_slot) c.N = read_i32(g, n_slot);
-        else if (!map) c.wide = false;
     }
 }
 
@@ -668,7 +666,6 @@ bool coarsen_level(bipart_graph *g, Level &f, Level &c, int policy, int32_t *siz
     }
     // N' is read with the contraction's sizes (one host round trip for the three)
     c.N = 0;
-    c.wide = f.wide;
     if (N > 0) {
         ProfScope ps("cmap", 24.0 * N, s);
         k_cmap<<<grid_for(N), kBlock, 0, s>>>(N, grp, gcid, f.nw(), f.cmap(), c.nw());

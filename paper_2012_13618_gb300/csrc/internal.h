@@ -143,7 +143,6 @@ struct ScanState {
 struct Level {
     int32_t N = 0, E = 0, P = 0;
     bool unit_hw = true;
-    bool wide = false;  // level 0 of its hierarchy has hyperedges of more than 256 pins
     Buf b_hoff, b_pins, b_hw, b_nw, b_noff, b_nadj, b_cmap, b_match;
     Buf b_tsh, b_tsn;  // tile-start tables of the hyperedge and incidence CSRs
     // A level built by the cluster tail (tail.cu) is a view into the tail's arena: hoff, pins,

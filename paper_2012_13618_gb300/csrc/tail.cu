@@ -1281,10 +1281,10 @@ namespace {
 // Where the tail may start (BIPART_TAIL_NODES and BIPART_TAIL_PINS, read once, lower or raise the limits).
 struct TailLimits {
     int nodes = kTailNodes;
-    int64_t pins = kTailStartPins, wide = kTailStartWide;
+    int64_t pins = kTailStartPins;
     TailLimits() {
         if (const char *env = std::getenv("BIPART_TAIL_NODES")) nodes = std::min(std::atoi(env), kTailNodes);
-        if (const char *env = std::getenv("BIPART_TAIL_PINS")) pins = wide = std::min<int64_t>(std::atoll(env), kTailMaxPins);
+        if (const char *env = std::getenv("BIPART_TAIL_PINS")) pins = std::min<int64_t>(std::atoll(env), kTailMaxPins);
     }
 };
 const TailLimits &tail_limits() {
@@ -1327,7 +1327,7 @@ bool tail_eligible(const Level &L, int max_new, int flags) {
     if (C <= 0) return false;
     if (flags & BIPART_FLAG_MERGE_PARALLEL) return false;  // the tail runs the paper's contraction
     if (max_new > kTailMaxLevels || L.N < 1) return false;
-    if (L.N > tail_limits().nodes || (int64_t)L.P > (L.wide ? tail_limits().wide : tail_limits().pins)) return false;
+    if (L.N > tail_limits().nodes || (int64_t)L.P > tail_limits().pins) return false;
     // every block's share of the chunk table fits its shared-memory copy
     return (tail_chunks(L.P) + C - 1) / C + 1 <= kTailMaxChunks;
 }

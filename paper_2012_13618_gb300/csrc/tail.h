@@ -19,14 +19,7 @@ constexpr int64_t kTailMaxPins = 4'000'000;  // ... and pins (its shared-memory 
 // on the server 56.5, 58.5, 57.4, 56.9, 61.7, 73.8 ms; one-shot 1,000 nodes 1177 us without, 740 us from
 // 10K up.  Above ~25K pins a level no longer fits one block's shared memory beside its nodes, and the
 // refinement's passes go back to L2.
-//
-// Where the input has hyperedges of more than 256 pins: kTailStartWide.  They are cut throughout, so every pass of
-// the one block handles all their pins, while on the cluster that refines larger levels they cost only when a
-// count passes 0, 1 or their last pins.  Netlists and row-nets of 5,000 to 13,000 nodes (30 of them), replays
-// from 25K, 17K and 10K pins: 0.97, 0.91, 0.89 of the time without a tail of their own before; first calls 0.88,
-// 0.88, 0.91.  Uniform hypergraphs (2 to 6 pins) of 7,000 nodes, first calls and replays: 800 and 690 us from
-// 25K, 1060 and 870 from 17K.
-constexpr int64_t kTailStartPins = 25'000, kTailStartWide = 17'000;
+constexpr int64_t kTailStartPins = 25'000;
 constexpr int kTailMaxLevels = 64;        // coarse levels one tail may build
 constexpr int kTailMaxCluster = 16;
 constexpr int kTailChunk = 2048;          // chunk boundaries of a level every this many pins

@@ -62,9 +62,8 @@ constexpr int kNT = kTailNodes;
 constexpr int kQ = kTailChunk;
 // Refinement: hyperedges of up to kThreadPins pins take a thread, up to kGroupPins eight lanes, wider ones a warp;
 // of a level whose pins are read through L2 up to kGroupPins a thread, wider ones a warp.  With up to 32 pins a
-// thread the longest loop was the pass (row-net level of 966 nodes, 20K pins: gains 26 us a pass, now 10, weighted
-// degrees 18 and 7; replays of row-nets of 2,000-8,000 nodes 1.1-1.4 times as long as on the grid, now 0.75-1.05);
-// all warps on the hyperedges of more than 256 pins gave nothing.
+// thread the longest loop was the pass (row-net level of 966 nodes, 20K pins: gains 26 us a pass, then 10); all warps
+// on the hyperedges of more than 256 pins gave nothing.
 constexpr int kThreadPins = 8, kGroupPins = 32;
 constexpr int kThreadDeg = 16;  // hyperedges up to this degree: one thread; above: one warp
 constexpr int kWarpDeg = 256;   // contraction: above this, the whole block (bitmap)
@@ -862,42 +861,49 @@ __device__ __forceinline__ void tiny_group(Pins pin, const int *hw, const uint8_
         if (sub + 8 * k < d) atomicAdd(out + u[k], on1 >> k & 1u ? x1 : x0);
 }
 
-// K hyperedges by a thread (d[k] = 0: none).  The first four pins of all of them are
-// handled straight-line, predicated: a loop per hyperedge costs a chain of shared-memory latencies and a
-// divergence each.
-template <int K, class Pins>
+// K hyperedges by a thread (d[k] = 0: none), their first kThreadPins pins straight-line and predicated: a loop per
+// hyperedge costs a chain of shared-memory latencies, and the lanes that left it at different times went on apart for
+// the rest of the pass (10 threads an instruction; thousand cycles a pass over 23K pins of 7,270 hyperedges 49, now
+// 15, over 20K of uniform 2 to 6 pins 10.5 and 9.6).  kLong: more pins may follow.  Converged warps.
+template <int K, bool kLong, class Pins>
 __device__ __forceinline__ void tiny_some(Pins pin, const int *hw, const uint8_t *side, int *out, bool gains,
                                           const int *e, const int *b, const int *d) {
-    int u[K][4];
+    int u[K][kThreadPins];
     unsigned on1[K];
 #pragma unroll
     for (int k = 0; k < K; ++k)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) u[k][i] = i < d[k] ? pin(b[k] + i) : 0;
+        for (int i = 0; i < kThreadPins; ++i) u[k][i] = i < d[k] ? pin(b[k] + i) : 0;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         on1[k] = 0;
         if (gains) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) on1[k] |= (i < d[k] ? (unsigned)side[u[k][i]] : 0u) << i;
+            for (int i = 0; i < kThreadPins; ++i) on1[k] |= (i < d[k] ? (unsigned)side[u[k][i]] : 0u) << i;
+        }
+        if constexpr (kLong) {
+            if (gains) {
+#pragma unroll 1
+                for (int i = kThreadPins; i < d[k]; ++i) on1[k] |= (unsigned)side[pin(b[k] + i)] << i;
+            }
+            __syncwarp();
         }
     }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        if (gains) {
-#pragma unroll 1
-            for (int i = 4; i < d[k]; ++i) on1[k] |= (unsigned)side[pin(b[k] + i)] << i;
-        }
         const int n1 = __popc(on1[k]), n0 = d[k] - n1;
-        if (gains && (n1 == 0 || n0 == 0)) continue;  // uncut: only -w_e, already in -D
-        const int w = hw && d[k] > 0 ? __ldcg(hw + e[k]) : 1;
+        const int m = gains && (n1 == 0 || n0 == 0) ? 0 : d[k];  // uncut: only -w_e, already in -D
+        const int w = hw && m > 0 ? __ldcg(hw + e[k]) : 1;
         // a pin alone on its side gets 2 w, the others w
         const int x1 = n1 == 1 ? 2 * w : w, x0 = gains && n0 == 1 ? 2 * w : w;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (i < d[k]) atomicAdd(out + u[k][i], on1[k] >> i & 1u ? x1 : x0);
+        for (int i = 0; i < kThreadPins; ++i)
+            if (i < m) atomicAdd(out + u[k][i], on1[k] >> i & 1u ? x1 : x0);
+        if constexpr (kLong) {
 #pragma unroll 1
-        for (int i = 4; i < d[k]; ++i) atomicAdd(out + pin(b[k] + i), on1[k] >> i & 1u ? x1 : x0);
+            for (int i = kThreadPins; i < m; ++i) atomicAdd(out + pin(b[k] + i), on1[k] >> i & 1u ? x1 : x0);
+            __syncwarp();
+        }
     }
 }
 
@@ -913,18 +919,19 @@ __device__ __noinline__ void tiny_edges(int sides) {
     if (s.lev.staged) {
         const StagedPins pin{reinterpret_cast<const uint16_t *>(tiny_at(s.lev.sp))};
         const uint16_t *so = reinterpret_cast<const uint16_t *>(tiny_at(s.lev.so));
-        constexpr int K = 4;
+        constexpr int K = 2;
 #pragma unroll 1
-        for (int e0 = threadIdx.x; e0 < E; e0 += K * kTT) {
+        for (int e0 = (int)(threadIdx.x & ~31u); e0 < E; e0 += K * kTT) {
             int e[K], b[K], d[K];
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                e[k] = e0 + k * kTT;
+                e[k] = e0 + lane + k * kTT;
                 b[k] = e[k] < E ? so[e[k]] : 0;
                 d[k] = e[k] < E ? so[e[k] + 1] - b[k] : 0;
                 if (d[k] > kThreadPins) d[k] = 0;
             }
-            tiny_some<K>(pin, hw, side, out, gains, e, b, d);
+            tiny_some<K, false>(pin, hw, side, out, gains, e, b, d);
+            __syncwarp();
         }
         __syncwarp();
         const uint16_t *list = reinterpret_cast<const uint16_t *>(tiny_at(s.lev.list));
@@ -959,7 +966,7 @@ __device__ __noinline__ void tiny_edges(int sides) {
                 todo[k] = __ballot_sync(0xffffffffu, d[k] > kGroupPins);
                 f[k] = d[k] > kGroupPins ? 0 : d[k];
             }
-            tiny_some<K>(pin, hw, side, out, gains, e, b, f);
+            tiny_some<K, true>(pin, hw, side, out, gains, e, b, f);
             __syncwarp();
 #pragma unroll 1
             for (int k = 0; k < K; ++k) {

@@ -846,7 +846,7 @@ __device__ __noinline__ void update_gains(bool own) {
     } else {
         n = __ldcg(&ls->rd[x.p].ents);
     }
-    const bool full = (long long)__ldcg(&ls->rd[x.solo ? 0 : x.p].inc) * kMoveCount > (long long)m.P;
+    const bool full = x.solo && (long long)__ldcg(&ls->rd[0].inc) * kMoveCount > (long long)m.P;
     LoopRound *rd = &ls->rd[x.solo ? 0 : x.p];
     // the histogram and the other round's lists are clear for the next selection
     if (!x.solo && x.r == x.C - 1) {

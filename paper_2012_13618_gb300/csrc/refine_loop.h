@@ -31,8 +31,8 @@ constexpr int kLoopSoloNodes = 4096;
 // nodes).  5M x 5M row-net, us of updates a level at P / 8, P / 32, P / 128: 1370 incidences a node 1779,
 // 2010, 2475; 2460 a node 2398, 1988, 2023; 4100 a node 2779, 2002, 1274; 5800 a node 3275, 1567, 1063.
 constexpr int kMoveFull = 8, kMoveFullHubs = 128, kHubDegree = 2048;
-// The cluster launch recounts above P / kMoveCount moved incidences: on levels of few nodes the updates' atomics meet on
-// the same gains (161 nodes, 110K pins: 39 us for the moves of a refinement selection; 150K-node netlist, its nodes'
+// On levels of at most kLoopSoloNodes nodes the cluster launch recounts above P / kMoveCount moved incidences: the
+// updates' atomics meet on the same gains, and no hyperedge is too wide for the warp that counts it (161 nodes, 110K pins: 39 us for the moves of a refinement selection; 150K-node netlist, its nodes'
 // high-fanout nets cut throughout, a bisection 1.69 ms, now 1.49; row-net of 30K nodes 1.83 and 1.71; at P / 16 1.5 %
 // slower, P / 4 the same).
 constexpr int kMoveCount = 8;

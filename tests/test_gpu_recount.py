@@ -1,6 +1,6 @@
 """Moves of a large share of a level's incidences: the cluster launch counts the gains afresh instead of updating them.
-Levels of few nodes and many pins, one selecting block and several, levels whose gains add up in shared memory and
-levels whose gains do not, wide and narrow hyperedges, weights.  Grid path alone (the coarse tail off) beside the
+Levels of few nodes and many pins up to the 4,096 nodes of one selecting block, and levels above, which go on
+updating; gains that add up in shared memory and gains that do not, wide and narrow hyperedges, weights.  Grid path alone (the coarse tail off) beside the
 default.  Integer arithmetic: identical to the oracle's."""
 import os
 import subprocess
@@ -29,9 +29,10 @@ def _cases():
     yield "few", _csr(60, [2, 3] * 6000, 1), 0.02, 2, 3
     yield "few_weighted", _csr(160, [2, 3, 5] * 8000, 2, hw_max=7, nw_max=6), 0.01, 2, 3
     yield "wide", _csr(400, [2] * 9000 + [31, 32, 33, 64, 400] * 40, 3, nw_max=3), 0.01, 3, 3
-    # all blocks select; 8 and 9 incidences a node (added up globally, in shared memory)
-    yield "shared_8", _csr(5000, [4] * 10_000, 4, nw_max=3), 0.02, 1, 4
-    yield "shared_9", _csr(5000, [4] * 10_000 + [5], 5, nw_max=3), 0.02, 1, 4
+    # 8 and 9 incidences a node (added up globally, in shared memory), the largest such level and the next
+    yield "sums_8", _csr(4096, [4] * 8192, 4, nw_max=3), 0.02, 0, 4
+    yield "sums_9", _csr(4096, [4] * 9000, 5, nw_max=3), 0.02, 0, 4
+    yield "above", _csr(4097, [4] * 9000, 8, nw_max=3), 0.02, 0, 4
     # more nodes than the shared-memory sums hold
     yield "many", _csr(20_000, [12] * 20_000, 6), 0.02, 1, 4
     # Algorithm 3 on a level of hubs

@@ -868,18 +868,33 @@ __device__ __forceinline__ void tiny_group(Pins pin, const int *hw, const uint8_
 template <int K, bool kLong, class Pins>
 __device__ __forceinline__ void tiny_some(Pins pin, const int *hw, const uint8_t *side, int *out, bool gains,
                                           const int *e, const int *b, const int *d) {
-    int u[K][kThreadPins];
+    static_assert(kThreadPins == 8, "two halves of four");
+    int u[K][kThreadPins], widest = 0;
     unsigned on1[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k)
+    for (int k = 0; k < K; ++k) widest = max(widest, d[k]);
+    const bool more = __any_sync(0xffffffffu, widest > 4);  // many levels have two pins a hyperedge throughout
 #pragma unroll
-        for (int i = 0; i < kThreadPins; ++i) u[k][i] = i < d[k] ? pin(b[k] + i) : 0;
+    for (int k = 0; k < K; ++k) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) u[k][i] = i < d[k] ? pin(b[k] + i) : 0;
+#pragma unroll
+        for (int i = 4; i < kThreadPins; ++i) u[k][i] = 0;
+        if (more) {
+#pragma unroll
+            for (int i = 4; i < kThreadPins; ++i) u[k][i] = i < d[k] ? pin(b[k] + i) : 0;
+        }
+    }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         on1[k] = 0;
         if (gains) {
 #pragma unroll
-            for (int i = 0; i < kThreadPins; ++i) on1[k] |= (i < d[k] ? (unsigned)side[u[k][i]] : 0u) << i;
+            for (int i = 0; i < 4; ++i) on1[k] |= (i < d[k] ? (unsigned)side[u[k][i]] : 0u) << i;
+            if (more) {
+#pragma unroll
+                for (int i = 4; i < kThreadPins; ++i) on1[k] |= (i < d[k] ? (unsigned)side[u[k][i]] : 0u) << i;
+            }
         }
         if constexpr (kLong) {
             if (gains) {
@@ -897,8 +912,13 @@ __device__ __forceinline__ void tiny_some(Pins pin, const int *hw, const uint8_t
         // a pin alone on its side gets 2 w, the others w
         const int x1 = n1 == 1 ? 2 * w : w, x0 = gains && n0 == 1 ? 2 * w : w;
 #pragma unroll
-        for (int i = 0; i < kThreadPins; ++i)
+        for (int i = 0; i < 4; ++i)
             if (i < m) atomicAdd(out + u[k][i], on1[k] >> i & 1u ? x1 : x0);
+        if (more) {
+#pragma unroll
+            for (int i = 4; i < kThreadPins; ++i)
+                if (i < m) atomicAdd(out + u[k][i], on1[k] >> i & 1u ? x1 : x0);
+        }
         if constexpr (kLong) {
 #pragma unroll 1
             for (int i = kThreadPins; i < m; ++i) atomicAdd(out + pin(b[k] + i), on1[k] >> i & 1u ? x1 : x0);
@@ -919,7 +939,7 @@ __device__ __noinline__ void tiny_edges(int sides) {
     if (s.lev.staged) {
         const StagedPins pin{reinterpret_cast<const uint16_t *>(tiny_at(s.lev.sp))};
         const uint16_t *so = reinterpret_cast<const uint16_t *>(tiny_at(s.lev.so));
-        constexpr int K = 2;
+        constexpr int K = 1;  // (2 the same within 1 %, 4 take the registers of the whole launch: 7 % slower)
 #pragma unroll 1
         for (int e0 = (int)(threadIdx.x & ~31u); e0 < E; e0 += K * kTT) {
             int e[K], b[K], d[K];
@@ -1288,10 +1308,10 @@ namespace {
 // Where the tail may start (BIPART_TAIL_NODES and BIPART_TAIL_PINS, read once, lower or raise the limits).
 struct TailLimits {
     int nodes = kTailNodes;
-    int64_t pins = kTailStartPins;
+    int64_t pins = kTailStartPins, pins_few = kTailStartFew;
     TailLimits() {
         if (const char *env = std::getenv("BIPART_TAIL_NODES")) nodes = std::min(std::atoi(env), kTailNodes);
-        if (const char *env = std::getenv("BIPART_TAIL_PINS")) pins = std::min<int64_t>(std::atoll(env), kTailMaxPins);
+        if (const char *env = std::getenv("BIPART_TAIL_PINS")) pins = pins_few = std::min<int64_t>(std::atoll(env), kTailMaxPins);
     }
 };
 const TailLimits &tail_limits() {
@@ -1334,7 +1354,7 @@ bool tail_eligible(const Level &L, int max_new, int flags) {
     if (C <= 0) return false;
     if (flags & BIPART_FLAG_MERGE_PARALLEL) return false;  // the tail runs the paper's contraction
     if (max_new > kTailMaxLevels || L.N < 1) return false;
-    if (L.N > tail_limits().nodes || (int64_t)L.P > tail_limits().pins) return false;
+    if (L.N > tail_limits().nodes || (int64_t)L.P > (L.N <= kTailFewNodes ? tail_limits().pins_few : tail_limits().pins)) return false;
     // every block's share of the chunk table fits its shared-memory copy
     return (tail_chunks(L.P) + C - 1) / C + 1 <= kTailMaxChunks;
 }

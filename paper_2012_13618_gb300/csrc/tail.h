@@ -13,14 +13,17 @@ namespace bp {
 constexpr int kTailThreads = 512;         // threads per block of the cluster
 constexpr int kTailNodes = 12288;         // largest level (nodes) the tail can start from
 constexpr int64_t kTailMaxPins = 4'000'000;  // ... and pins (its shared-memory chunk table)
-// Default start: the first level of at most this many pins.  Swept as the start (10K, 25K, 35K, 45K pins), geometric
-// means over 78 netlists, row-nets and uniform hypergraphs of 2,000 to 150,000 nodes, of the time without a tail in
-// replays and with one from 70K pins in first calls (a cluster refined it): first calls 0.83, 0.74, 0.72, 0.71, replays
-// 0.80, 0.77, 0.78, 0.79; 10K-node uniform replays 782, 730, 811 us from 25K, 35K, 45K; 16-way parts
-// of a 250K-node netlist 12.37, 12.36, 12.47 ms from 25K, 35K, 45K; a mix of 12 graphs on the server 49.4, 48.8, 48.5.
+// Default start: the first level of at most kTailStartPins pins, or of kTailStartFew on levels of at most kTailFewNodes
+// nodes (with more, the one block's selections cost more than the grid's launches: uniform hypergraph of 7,000 nodes
+// and 28K pins, replays 642 and 665 us from its second level and its first).  Swept as the start (10K, 25K, 35K, 45K
+// pins whatever the nodes), geometric means over 80 netlists, row-nets and uniform hypergraphs of 2,000 to 150,000
+// nodes, of the times without a tail in replays and with one of a whole cluster from 70K pins in first calls: first
+// calls 0.83, 0.74, 0.72, 0.72, replays 0.81, 0.78, 0.79, 0.80; 10K-node uniform replays 782, 730, 811 us from 25K, 35K,
+// 45K; 16-way parts of a 250K-node netlist 12.37, 12.36, 12.47 ms; a mix of 12 graphs on the server 49.4, 48.8, 48.5.
 // Above ~35K pins a level no longer fits one block's shared memory beside its nodes, and the refinement's passes go
 // back to L2.
-constexpr int64_t kTailStartPins = 35'000;
+constexpr int64_t kTailStartPins = 25'000, kTailStartFew = 35'000;
+constexpr int kTailFewNodes = kTailNodes / 2;
 constexpr int kTailMaxLevels = 64;        // coarse levels one tail may build
 constexpr int kTailMaxCluster = 16;
 constexpr int kTailChunk = 2048;          // chunk boundaries of a level every this many pins

@@ -1,5 +1,5 @@
-"""The coarse tail takes hypergraphs of up to 35,000 pins and 12,288 nodes whole, with the pins in shared memory and
-without; one pin or node more is coarsened on the grid first.  Integer arithmetic: identical to the oracle's."""
+"""The coarse tail takes hypergraphs of up to 35,000 pins and 6,144 nodes, or 25,000 pins and 12,288 nodes, whole, with the
+pins in shared memory and without; one pin or node more is coarsened on the grid first.  Integer arithmetic: identical to the oracle's."""
 import numpy as np
 import pytest
 
@@ -8,8 +8,9 @@ import oracle
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("N,pins,whole", [(3000, 35_000, True), (3000, 35_001, False), (12_288, 35_000, True),
-                                          (12_289, 34_999, False)])
+@pytest.mark.parametrize("N,pins,whole", [(3000, 35_000, True), (3000, 35_001, False), (6144, 35_000, True),
+                                          (6145, 25_001, False), (6145, 25_000, True), (12_288, 25_000, True),
+                                          (12_289, 24_999, False)])
 def test_tail_limits_match_oracle(N, pins, whole):
     import paper_2012_13618_gb300 as bp
     rng = np.random.default_rng(pins + N)

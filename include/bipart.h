@@ -46,7 +46,8 @@ typedef struct bipart_graph *bipart_handle;
 
 /* Optional device allocator used for every device buffer the library owns (for example the
  * caching allocator of a framework).  alloc returns NULL on failure; both receive the handle's
- * stream.  With no allocator set the library uses cudaMallocAsync / cudaFreeAsync on that stream.
+ * stream.  Pointers may have any alignment (the library aligns its arrays inside the allocation).
+ * With no allocator set the library uses cudaMallocAsync / cudaFreeAsync on that stream.
  * Applies to allocations made after the call; pass NULLs to restore the default.  A buffer is
  * always freed by the allocator that made it.  The batch call, the server and nested k-way
  * allocate from several host threads at once: the functions must be thread-safe, and an

@@ -32,17 +32,17 @@ constexpr int kLoopSoloNodes = 4096;
 // 2010, 2475; 2460 a node 2398, 1988, 2023; 4100 a node 2779, 2002, 1274; 5800 a node 3275, 1567, 1063.
 constexpr int kMoveFull = 8, kMoveFullHubs = 128, kHubDegree = 2048;
 // On levels of at most kLoopSoloNodes nodes the cluster launch recounts above P / kMoveCount moved incidences: the
-// updates' atomics meet on the same gains, and no hyperedge is too wide for the warp that counts it (161 nodes, 110K pins: 39 us for the moves of a refinement selection; 150K-node netlist, its nodes'
-// high-fanout nets cut throughout, a bisection 1.69 ms, now 1.49; row-net of 30K nodes 1.83 and 1.71; at P / 16 1.5 %
-// slower, P / 4 the same).
+// updates' atomics meet on the same gains, and no hyperedge is too wide for the warp that counts it (161 nodes, 110K
+// pins: 39 us for the moves of a refinement selection; 150K-node netlist whose high-fanout nets are cut throughout 1.69
+// ms a bisection, then 1.49; row-net of 30K nodes 1.83 and 1.71; at P / 16 1.5 % slower, at P / 4 the same).
 constexpr int kMoveCount = 8;
 
 // Refinement selections run on the whole grid on levels of more than kGridSelLarge nodes, and of more than
-// kGridSelNodes nodes and kLoopAlonePins pins where the coarser level has kGridSelRatio times fewer (its sides are a rough start, so many
-// nodes move); the others stay in the cluster launch, whose steps are cheaper when few do.  Bisections, cluster
-// and grid: 5M-node row-net 55.8 and 53.6 ms; 155K-node netlist merged by its largest nets (HDH, four iterations)
-// 1069 and 906 us, 600K-node row-net alike 2910 and 2658; 1M-node netlist 2753 and 2797, kept 500K-node
-// hierarchy refined 2314 and 2521.
+// kGridSelNodes nodes and kLoopAlonePins pins where the coarser level has kGridSelRatio times fewer nodes (its sides
+// are a rough start, so many nodes move); the others stay in the cluster launch, whose steps are cheaper when few do.
+// Bisections, cluster and grid: 5M-node row-net 55.8 and 53.6 ms; 155K-node netlist merged by its largest nets (HDH,
+// four iterations) 1069 and 906 us, 600K-node row-net alike 2910 and 2658; 1M-node netlist 2753 and 2797, kept
+// 500K-node hierarchy refined 2314 and 2521.
 constexpr int kGridSelNodes = 1 << 17, kGridSelLarge = 1 << 21, kGridSelRatio = 8;
 
 // What one selection leaves for the update after it; two are used in turn.
